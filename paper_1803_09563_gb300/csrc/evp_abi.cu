@@ -403,17 +403,21 @@ int prepare_helmholtz(evp_state* s, double dt) {
     const std::vector<double> lx = lam(g.nx, nxh, dx), lz = lam(g.nz, g.nz / 2 + 1, dz);
     const double mu_s = s->prm.beta / s->prm.Re;
     static const double RK3_ALPHA_H[3] = {4.0 / 15.0, 1.0 / 15.0, 1.0 / 6.0};
+    // on the state's stream: a copy on the legacy stream may still be on its way to the
+    // device when cudaMemcpy returns (pageable memory is only staged by then), and a
+    // non-blocking stream does not wait for it
     CK(cudaStreamSynchronize(s->st));
     for (int k = 0; k < 3; ++k)
         for (int q = 0; q < 2; ++q) {
             const std::vector<double> M = helmholtz_table(g.ny, g.nz, nxh, dy, lx, lz, RK3_ALPHA_H[k] * dt * mu_s, q == 1);
             if (s->fp32 && !s->prm.thomas_fp64) {
                 const std::vector<float> F = thomas_table_ds(M);
-                CK(cudaMemcpy(s->helm[k][q], F.data(), F.size() * sizeof(float), cudaMemcpyHostToDevice));
+                CK(cudaMemcpyAsync(s->helm[k][q], F.data(), F.size() * sizeof(float), cudaMemcpyHostToDevice, s->st));
             } else {
-                CK(cudaMemcpy(s->helm[k][q], M.data(), M.size() * sizeof(double), cudaMemcpyHostToDevice));
+                CK(cudaMemcpyAsync(s->helm[k][q], M.data(), M.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
             }
         }
+    CK(cudaStreamSynchronize(s->st));
     s->helm_dt = dt;
     return EVP_OK;
 }
@@ -1182,18 +1186,20 @@ extern "C" int evp_set_particles(evp_state* s, int n, const double* desc, int it
     s->i_int = s->i_dens + n;
     s->i_owner = reinterpret_cast<int*>(s->i_int + 12 * n);
     s->i_start = s->i_owner + nl;
-    CK(cudaMemcpy(s->i_off, off.data(), off.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s->i_dvl, dvl.data(), dvl.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s->i_centre, centre.data(), centre.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s->i_vel, vel.data(), vel.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s->i_omg, omg.data(), omg.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemset(s->i_Facc, 0, 3 * nl * sizeof(double)));
-    CK(cudaMemset(s->i_force, 0, 6 * n * sizeof(double)));
-    CK(cudaMemcpy(s->i_rad, rad.data(), rad.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s->i_dens, dens.data(), dens.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemset(s->i_int, 0, 12 * n * sizeof(double)));
-    CK(cudaMemcpy(s->i_owner, owner.data(), owner.size() * sizeof(int), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(s->i_start, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice));
+    // on the state's stream, whose kernels read the arrays (see prepare_helmholtz)
+    CK(cudaMemcpyAsync(s->i_off, off.data(), off.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemcpyAsync(s->i_dvl, dvl.data(), dvl.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemcpyAsync(s->i_centre, centre.data(), centre.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemcpyAsync(s->i_vel, vel.data(), vel.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemcpyAsync(s->i_omg, omg.data(), omg.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemsetAsync(s->i_Facc, 0, 3 * nl * sizeof(double), s->st));
+    CK(cudaMemsetAsync(s->i_force, 0, 6 * n * sizeof(double), s->st));
+    CK(cudaMemcpyAsync(s->i_rad, rad.data(), rad.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemcpyAsync(s->i_dens, dens.data(), dens.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemsetAsync(s->i_int, 0, 12 * n * sizeof(double), s->st));
+    CK(cudaMemcpyAsync(s->i_owner, owner.data(), owner.size() * sizeof(int), cudaMemcpyHostToDevice, s->st));
+    CK(cudaMemcpyAsync(s->i_start, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice, s->st));
+    CK(cudaStreamSynchronize(s->st));
     s->n_part = n;
     s->n_lag = (int)nl;
     s->ibm_iters = iters;

@@ -258,7 +258,13 @@ int prepare(evp_batch* b) {
         }
         b->work_cap = cap;
     }
-    if (!work.empty()) BCK(cudaMemcpy(b->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    if (!work.empty()) {
+        // on the batch's stream: a plain cudaMemcpy of pageable memory may return while
+        // the copy is still on its way, on a stream that the batch's (non-blocking) one
+        // does not wait for, and the first step would walk the old list
+        BCK(cudaMemcpyAsync(b->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, b->st));
+        BCK(cudaStreamSynchronize(b->st));
+    }
     b->dirty = false;
     return EVP_OK;
 }
