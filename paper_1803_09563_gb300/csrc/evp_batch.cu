@@ -77,12 +77,16 @@ int default_kz(int nx, int ny, int nz, int tx, int ty, int per_sm) {
     return (nz + chunks - 1) / chunks;
 }
 
+StressShape shape_of(const evp_grid& g, int precision) {
+    return precision == EVP_FP32 ? stress_shape<float>(g.nx, g.ny) : stress_shape<double>(g.nx, g.ny);
+}
+
 evp_tile_config default_config(const evp_grid& g, int precision) {
     const bool f32 = precision == EVP_FP32;
     evp_tile_config c;
     c.stress_ctas_per_sm = f32 ? stress_ctas_per_sm<float>() : stress_ctas_per_sm<double>();
     c.momentum_ctas_per_sm = f32 ? momentum_ctas_per_sm<float>() : momentum_ctas_per_sm<double>();
-    c.stress_kz = default_kz(g.nx, g.ny, g.nz, stress_tile_x(), stress_tile_y(), c.stress_ctas_per_sm);
+    c.stress_kz = f32 ? stress_planes<float>(g.nx, g.ny, g.nz) : stress_planes<double>(g.nx, g.ny, g.nz);
     c.momentum_kz = default_kz(g.nx, g.ny, g.nz, momentum_tile_x(), momentum_tile_y(), c.momentum_ctas_per_sm);
     c.fft_cols = f32 ? 16 : 8;
     return c;
@@ -140,6 +144,7 @@ struct evp_batch_s {
         int model = 0;
         bool vec = true;
         int work_off = 0, nwork = 0, ctas = 0;
+        size_t smem = 0;        // stress launches: dynamic shared memory
     };
     std::vector<Launch> stress, momentum;
     struct Group {
@@ -230,11 +235,14 @@ int prepare(evp_batch* b) {
         int per_sm = 1;
         for (int gi = 0; gi < (int)l.idx.size(); ++gi) {
             const auto& mb = b->m[l.idx[gi]];
-            add_work(work, gi, mb.s->g, stress_tile_x(), stress_tile_y(), mb.cfg.stress_kz);
+            const StressShape sh = shape_of(mb.s->g, b->precision);
+            add_work(work, gi, mb.s->g, sh.tw, sh.th, mb.cfg.stress_kz);
             per_sm = std::max(per_sm, mb.cfg.stress_ctas_per_sm);
+            l.smem = std::max(l.smem, b->precision == EVP_FP32 ? stress_smem<float>(mb.s->g.nx, mb.s->g.ny)
+                                                               : stress_smem<double>(mb.s->g.nx, mb.s->g.ny));
         }
         l.nwork = (int)work.size() - l.work_off;
-        l.ctas = per_sm * sms;
+        l.ctas = per_sm * sms * (b->precision == EVP_FP32 ? stress_cta_factor<float>() : stress_cta_factor<double>());
     }
     for (auto& l : b->momentum) {
         l.work_off = (int)work.size();
@@ -295,6 +303,9 @@ int step_direct(evp_batch* b) {
                 M.g = geo_of<T>(s);
                 M.mc = s->mc;
                 M.kz = mb.cfg.stress_kz;
+                const StressShape sh = shape_of(s->g, b->precision);
+                M.tw = sh.tw;
+                M.th = sh.th;
                 StressArgs<T>& a = M.a;
                 const int cu = s->cu, cb = s->cb;
                 a.U = static_cast<const T*>(s->U[cu]);
@@ -316,7 +327,7 @@ int step_direct(evp_batch* b) {
                 a.mu_p1 = a.mu_p2 = T(0);
             }
             const cudaError_t e =
-                launch_stress_batch<T>(*sp, l.model, mode, l.vec, b->d_work + l.work_off, l.nwork, l.ctas, b->st);
+                launch_stress_batch<T>(*sp, l.model, mode, l.vec, b->d_work + l.work_off, l.nwork, l.ctas, l.smem, b->st);
             if (e != cudaSuccess) return bcuda(e, "batched stress kernel");
         }
         // ---- S3: momentum predictor (Eq. rk3) with the summed stress

@@ -389,6 +389,7 @@ struct StressMember {
     ModelConst mc;
     StressArgs<T> a;
     int kz;            // z planes per work item
+    int tw, th;        // tile shape (stress_shape)
 };
 template <typename T>
 struct StressBatch {
@@ -600,16 +601,28 @@ cudaError_t launch_momentum(const Geo<T>& g, const ModelConst& mc, const Momentu
 // Batched launches.  work: device list of int4 (member, tile x, tile y, z chunk);
 // ctas: size of the persistent grid.  The stress batch holds members of one model
 // and one staging kind (vec: nx * sizeof(T) % 16 == 0); mode 1, 2, 3 as the
-// update modes of the stress kernel.  The momentum batch reads the summed stress.
+// update modes of the stress kernel; smem: the largest stress_smem of the members.
+// The momentum batch reads the summed stress.
 template <typename T>
 cudaError_t launch_stress_batch(const StressBatch<T>& p, int model, int mode, bool vec, const int4* work, int nwork,
-                                int ctas, cudaStream_t st);
+                                int ctas, size_t smem, cudaStream_t st);
 template <typename T>
 cudaError_t launch_momentum_batch(const MomentumBatch<T>& p, bool vec, const int4* work, int nwork, int ctas,
                                   cudaStream_t st);
-// tiles and resident CTAs per SM of the z-marching kernels
-int stress_tile_x();
-int stress_tile_y();
+// tiles and resident CTAs per SM of the z-marching kernels.  The stress kernel's tile
+// is 32 x 8 in single precision and depends on the grid in double precision, where a
+// counted CTA per SM is two launched ones of half the threads (stress_cta_factor).
+struct StressShape {
+    int tw, th;
+};
+template <typename T>
+StressShape stress_shape(int nx, int ny);
+template <typename T>
+int stress_planes(int nx, int ny, int nz);   // z planes per CTA of a single-state launch
+template <typename T>
+size_t stress_smem(int nx, int ny);
+template <typename T>
+int stress_cta_factor();
 int momentum_tile_x();
 int momentum_tile_y();
 template <typename T>

@@ -5,8 +5,9 @@
 //      [+ kappa_ad lap B where det B < 0 or, FENE-P, tr B >= 0.95 L^2  (Sec. 3.1)]
 // B^k = B^{k-1} + dt (zeta^k RT^{k-1} + xi^k RT^{k-2})            (Eq. rk3tau)
 //
-// z-marching tiles: see the kernel for the data staging.  The kernel template is
-// instantiated once per precision, in k_stress_f32.cu and k_stress_f64.cu.
+// z-marching tiles: see the kernel for the data staging.  Single precision
+// (instantiated in k_stress_f32.cu); double precision, whose bound is another, is in
+// k_stress_f64.cu.
 #pragma once
 #include <cfloat>
 
@@ -104,10 +105,7 @@ struct StressSmem {
 template <typename T>
 __device__ __forceinline__ void cp_async(T* smem, const T* gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    if (sizeof(T) == 4)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
@@ -281,21 +279,12 @@ __device__ __forceinline__ void stress_tile(const Geo<T>& g, const ModelConst& m
     const T* vel[3] = {a.U, a.V, a.W};
     // E elements from global (one 16-byte vector) into shared, times fac (+1, -1, 0)
     auto copy_scaled = [&](T* dst, const T* src, int fac) {
-        if (sizeof(T) == 4) {
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (fac) {
-                v = __ldg(reinterpret_cast<const float4*>(src));
-                v.x = -v.x; v.y = -v.y; v.z = -v.z; v.w = -v.w;
-            }
-            *reinterpret_cast<float4*>(dst) = v;
-        } else {
-            double2 v = make_double2(0.0, 0.0);
-            if (fac) {
-                v = __ldg(reinterpret_cast<const double2*>(src));
-                v.x = -v.x; v.y = -v.y;
-            }
-            *reinterpret_cast<double2*>(dst) = v;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (fac) {
+            v = __ldg(reinterpret_cast<const float4*>(src));
+            v.x = -v.x; v.y = -v.y; v.z = -v.z; v.w = -v.w;
         }
+        *reinterpret_cast<float4*>(dst) = v;
     };
     // velocity plane kk (unwrapped index) into ring slot kk mod 4
     auto fetch_vel = [&](int kk) {
@@ -457,8 +446,7 @@ __device__ __forceinline__ void stress_tile(const Geo<T>& g, const ModelConst& m
             av = T(0);
         } else if (MODEL == EVP_FENE_P) {
             const T tr = b0[0] + b0[3] + b0[5];
-            if (sizeof(T) == 4) F = kL2 * T(rcp_approx(float(kL2 - tr)));
-            else F = kL2 / (kL2 - tr);
+            F = kL2 * rcp_approx(kL2 - tr);
             av = kaf;
         } else if (MODEL == EVP_SARAMITO) {
             T gm = kgm;
@@ -475,19 +463,12 @@ __device__ __forceinline__ void stress_tile(const Geo<T>& g, const ModelConst& m
             const T d0 = t[0] - tr3, d3 = t[3] - tr3, d5 = t[5] - tr3;
             const T mag2 = T(0.5) * (d0 * d0 + d3 * d3 + d5 * d5) + t[1] * t[1] + t[2] * t[2] + t[4] * t[4];
             const T tyv = kty;
-            if (sizeof(T) == 4) {
-                // F = max(0, 1 - tau_y/|tau^d|) with the approximate reciprocal square
-                // root instruction; tau_y = 0 is exactly Oldroyd-B (F = 1)
-                float rs;
-                asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(float(mag2)));
-                const T f = T(1) - tyv * T(rs);
-                F = tyv > T(0) ? (mag2 > T(0) && f > T(0) ? f : T(0)) : T(1);
-            } else if (mag2 > T(0)) {
-                const T f = T(1) - tyv / sqrt(mag2);
-                F = f > T(0) ? f : T(0);
-            } else {
-                F = tyv > T(0) ? T(0) : T(1);
-            }
+            // F = max(0, 1 - tau_y/|tau^d|) with the approximate reciprocal square
+            // root instruction; tau_y = 0 is exactly Oldroyd-B (F = 1)
+            float rs;
+            asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(mag2));
+            const T f = T(1) - tyv * rs;
+            F = tyv > T(0) ? (mag2 > T(0) && f > T(0) ? f : T(0)) : T(1);
             av = F;
         }
 
@@ -514,32 +495,20 @@ __device__ __forceinline__ void stress_tile(const Geo<T>& g, const ModelConst& m
 #pragma unroll
         for (int n = 0; n < 6; ++n) zo[n] = ((zpos ? k - 3 + n : k + 3 - n) & 7) * (6 * NT) + tid;
         T bn[6], advc[6];
-        if constexpr (sizeof(T) == 4) {
-            // single precision: the components in pairs (xx, xy), (xz, yy), (yz, zz),
-            // which share the upwind side and |u|/h, on the packed f32x2 instructions
+        // the components in pairs (xx, xy), (xz, yy), (yz, zz), which share the upwind
+        // side and |u|/h, on the packed f32x2 instructions
 #pragma unroll
-            for (int p = 0; p < 3; ++p) {
-                const float* P0 = Bk + (2 * p) * BPL;
-                const float* P1 = P0 + BPL;
-                auto at = [&](int off) { return make_float2(P0[ob + off], P1[ob + off]); };
-                auto zz = [&](int n) { return make_float2(Nf[zo[n] + (2 * p) * NT], Nf[zo[n] + (2 * p + 1) * NT]); };
-                float2 s = upwind_term2(splat2(vx_), at(-3 * sx), at(-2 * sx), at(-sx), at(0), at(sx), at(2 * sx));
-                s = add2(s, upwind_term2(splat2(vy_), at(-3 * syw), at(-2 * syw), at(-syw), at(0), at(syw), at(2 * syw)));
-                // z stencil from the ring
-                s = add2(s, upwind_term2(splat2(vz_), zz(0), zz(1), zz(2), zz(3), zz(4), zz(5)));
-                advc[2 * p] = s.x;
-                advc[2 * p + 1] = s.y;
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                const T* P = Bk + c * BPL;
-                T adv = upwind_term(vx_, P[ob - 3 * sx], P[ob - 2 * sx], P[ob - sx], P[ob], P[ob + sx], P[ob + 2 * sx]);
-                adv += upwind_term(vy_, P[ob - 3 * syw], P[ob - 2 * syw], P[ob - syw], P[ob], P[ob + syw], P[ob + 2 * syw]);
-                // z stencil from the ring
-                advc[c] = adv + upwind_term(vz_, Nf[zo[0] + c * NT], Nf[zo[1] + c * NT], Nf[zo[2] + c * NT], b0[c],
-                                            Nf[zo[4] + c * NT], Nf[zo[5] + c * NT]);
-            }
+        for (int p = 0; p < 3; ++p) {
+            const float* P0 = Bk + (2 * p) * BPL;
+            const float* P1 = P0 + BPL;
+            auto at = [&](int off) { return make_float2(P0[ob + off], P1[ob + off]); };
+            auto zz = [&](int n) { return make_float2(Nf[zo[n] + (2 * p) * NT], Nf[zo[n] + (2 * p + 1) * NT]); };
+            float2 s = upwind_term2(splat2(vx_), at(-3 * sx), at(-2 * sx), at(-sx), at(0), at(sx), at(2 * sx));
+            s = add2(s, upwind_term2(splat2(vy_), at(-3 * syw), at(-2 * syw), at(-syw), at(0), at(syw), at(2 * syw)));
+            // z stencil from the ring
+            s = add2(s, upwind_term2(splat2(vz_), zz(0), zz(1), zz(2), zz(3), zz(4), zz(5)));
+            advc[2 * p] = s.x;
+            advc[2 * p + 1] = s.y;
         }
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
@@ -613,7 +582,7 @@ __device__ __forceinline__ void stress_tile(const Geo<T>& g, const ModelConst& m
 }
 
 template <typename T, int MODEL, int MODE, bool DIFF, bool VEC>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(NT, 2)
 k_stress(const Geo<T> g, const ModelConst mc, const StressArgs<T> a, int kz_chunk) {
     pdl_wait();
     pdl_trigger();
@@ -625,7 +594,7 @@ k_stress(const Geo<T> g, const ModelConst mc, const StressArgs<T> a, int kz_chun
 // z chunk) over the members of a batch, whose grids may differ; the members'
 // arguments sit in the kernel's parameter space.
 template <typename T, int MODEL, int MODE, bool DIFF, bool VEC>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(NT, 2)
 k_stress_batch(const __grid_constant__ StressBatch<T> p, const int4* __restrict__ work, int nwork) {
     extern __shared__ __align__(16) unsigned char smraw[];
     for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
@@ -681,10 +650,9 @@ cudaError_t launch_stress_v(const Geo<T>& g, const ModelConst& mc, const StressA
 // model, one mode and one staging kind, the caller groups them so).
 template <typename T>
 cudaError_t launch_stress_batch(const StressBatch<T>& p, int model, int mode, bool vec, const int4* work, int nwork,
-                                int ctas, cudaStream_t st) {
+                                int ctas, size_t smem, cudaStream_t st) {
     if (nwork <= 0) return cudaSuccess;
     dim3 block(TX, TY, 1);
-    const size_t smem = sizeof(StressSmem<T>);
     const dim3 grid(ctas < nwork ? ctas : nwork);
     auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -710,29 +678,32 @@ cudaError_t launch_stress_batch(const StressBatch<T>& p, int model, int mode, bo
 
 // resident CTAs of the stress kernel per SM (shared memory and registers)
 template <typename T>
-int stress_ctas_per_sm() { return sizeof(T) == 4 ? 2 : 1; }
+int stress_ctas_per_sm() { return 2; }
+template <typename T>
+int stress_cta_factor() { return 1; }
+template <typename T>
+StressShape stress_shape(int, int) { return {TX, TY}; }
+template <typename T>
+size_t stress_smem(int, int) { return sizeof(StressSmem<T>); }
+
+// z planes per CTA: about four waves of CTAs over all SMs (two CTAs per SM); small
+// grids go down to one plane per CTA so that every SM works
+template <typename T>
+int stress_planes(int nx, int ny, int nz) {
+    const int tiles = ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
+    int chunks = (4 * 152 * 2 + tiles - 1) / tiles;
+    chunks = chunks > nz ? nz : chunks;
+    return (nz + chunks - 1) / chunks;
+}
 
 template <typename T>
 cudaError_t launch_stress(const Geo<T>& g, const ModelConst& mc, const StressArgs<T>& a,
                           cudaStream_t st, const TimingHook& th) {
-    // z chunks: about four waves of CTAs over all SMs (two CTAs per SM in FP32,
-    // one in FP64); small grids go down to one plane per CTA so that every SM works
-    const int tiles = ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
-    const int per_sm = sizeof(T) == 4 ? 2 : 1;
-    int chunks = (4 * 152 * per_sm + tiles - 1) / tiles;
-    chunks = chunks > g.nz ? g.nz : chunks;
-    const int kz = (g.nz + chunks - 1) / chunks;
-    chunks = (g.nz + kz - 1) / kz;
-    dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, chunks);
+    const int kz = stress_planes<T>(g.nx, g.ny, g.nz);
+    dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + kz - 1) / kz);
     th.b(K_STRESS);
-    cudaError_t e;
-    // 16-byte chunks need whole chunks per row: always so in FP64 (nx is even)
-    if constexpr (sizeof(T) == 8) {
-        e = launch_stress_v<T, true>(g, mc, a, st, grid, kz, th.pdl);
-    } else {
-        e = (g.nx * sizeof(T)) % 16 == 0 ? launch_stress_v<T, true>(g, mc, a, st, grid, kz, th.pdl)
-                                         : launch_stress_v<T, false>(g, mc, a, st, grid, kz, th.pdl);
-    }
+    const cudaError_t e = (g.nx * sizeof(T)) % 16 == 0 ? launch_stress_v<T, true>(g, mc, a, st, grid, kz, th.pdl)
+                                                       : launch_stress_v<T, false>(g, mc, a, st, grid, kz, th.pdl);
     if (e != cudaSuccess) return e;
     th.e(K_STRESS);
     return cudaGetLastError();
