@@ -69,14 +69,6 @@ CfgKey cfg_key(const evp_grid& g, int precision, int model) {
     return CfgKey(g.nx, g.ny, g.nz, g.walls_y ? 1 : 0, precision, model);
 }
 
-// z planes per work item of the single-state launches: about four waves of CTAs
-int default_kz(int nx, int ny, int nz, int tx, int ty, int per_sm) {
-    const int tiles = ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
-    int chunks = (4 * 152 * per_sm + tiles - 1) / tiles;
-    chunks = chunks > nz ? nz : chunks;
-    return (nz + chunks - 1) / chunks;
-}
-
 StressShape shape_of(const evp_grid& g, int precision) {
     return precision == EVP_FP32 ? stress_shape<float>(g.nx, g.ny) : stress_shape<double>(g.nx, g.ny);
 }
@@ -87,7 +79,7 @@ evp_tile_config default_config(const evp_grid& g, int precision) {
     c.stress_ctas_per_sm = f32 ? stress_ctas_per_sm<float>() : stress_ctas_per_sm<double>();
     c.momentum_ctas_per_sm = f32 ? momentum_ctas_per_sm<float>() : momentum_ctas_per_sm<double>();
     c.stress_kz = f32 ? stress_planes<float>(g.nx, g.ny, g.nz) : stress_planes<double>(g.nx, g.ny, g.nz);
-    c.momentum_kz = default_kz(g.nx, g.ny, g.nz, momentum_tile_x(), momentum_tile_y(), c.momentum_ctas_per_sm);
+    c.momentum_kz = f32 ? momentum_planes<float>(g.nx, g.ny, g.nz) : momentum_planes<double>(g.nx, g.ny, g.nz);
     c.fft_cols = f32 ? 16 : 8;
     return c;
 }
@@ -177,9 +169,9 @@ void drop_graphs(evp_batch* b) {
 bool has_vec(const evp_state* s) { return ((size_t)s->g.nx * s->elt) % 16 == 0; }
 
 // Work list entries (member index within its launch, tile x, tile y, z chunk) of
-// a z-marching kernel with tx x ty tiles and kz planes per item.
-void add_work(std::vector<int4>& w, int gi, const evp_grid& g, int tx, int ty, int kz) {
-    const int nbx = (g.nx + tx - 1) / tx, nby = (g.ny + ty - 1) / ty, nbz = (g.nz + kz - 1) / kz;
+// a z-marching kernel with nbx x nby tiles and kz planes per item.
+void add_work(std::vector<int4>& w, int gi, const evp_grid& g, int nbx, int nby, int kz) {
+    const int nbz = (g.nz + kz - 1) / kz;
     for (int bz = 0; bz < nbz; ++bz)
         for (int by = 0; by < nby; ++by)
             for (int bx = 0; bx < nbx; ++bx) w.push_back(make_int4(gi, bx, by, bz));
@@ -236,7 +228,8 @@ int prepare(evp_batch* b) {
         for (int gi = 0; gi < (int)l.idx.size(); ++gi) {
             const auto& mb = b->m[l.idx[gi]];
             const StressShape sh = shape_of(mb.s->g, b->precision);
-            add_work(work, gi, mb.s->g, sh.tw, sh.th, mb.cfg.stress_kz);
+            add_work(work, gi, mb.s->g, (mb.s->g.nx + sh.tw - 1) / sh.tw, (mb.s->g.ny + sh.th - 1) / sh.th,
+                     mb.cfg.stress_kz);
             per_sm = std::max(per_sm, mb.cfg.stress_ctas_per_sm);
             l.smem = std::max(l.smem, b->precision == EVP_FP32 ? stress_smem<float>(mb.s->g.nx, mb.s->g.ny)
                                                                : stress_smem<double>(mb.s->g.nx, mb.s->g.ny));
@@ -249,11 +242,13 @@ int prepare(evp_batch* b) {
         int per_sm = 1;
         for (int gi = 0; gi < (int)l.idx.size(); ++gi) {
             const auto& mb = b->m[l.idx[gi]];
-            add_work(work, gi, mb.s->g, momentum_tile_x(), momentum_tile_y(), mb.cfg.momentum_kz);
+            const MomentumTiles t = b->precision == EVP_FP32 ? momentum_tiles<float>(mb.s->g.nx, mb.s->g.ny)
+                                                             : momentum_tiles<double>(mb.s->g.nx, mb.s->g.ny);
+            add_work(work, gi, mb.s->g, t.x, t.y, mb.cfg.momentum_kz);
             per_sm = std::max(per_sm, mb.cfg.momentum_ctas_per_sm);
         }
         l.nwork = (int)work.size() - l.work_off;
-        l.ctas = per_sm * sms;
+        l.ctas = sms * (b->precision == EVP_FP32 ? momentum_resident<float>(per_sm) : momentum_resident<double>(per_sm));
     }
     if (work.size() > b->work_cap) {
         if (b->d_work) cudaFree(b->d_work);

@@ -623,8 +623,16 @@ template <typename T>
 size_t stress_smem(int nx, int ny);
 template <typename T>
 int stress_cta_factor();
-int momentum_tile_x();
-int momentum_tile_y();
+// tiles of a plane and z planes per CTA of the momentum kernel
+struct MomentumTiles {
+    int x, y;
+};
+template <typename T>
+MomentumTiles momentum_tiles(int nx, int ny);
+template <typename T>
+int momentum_planes(int nx, int ny, int nz);
+template <typename T>
+int momentum_resident(int counted);          // CTAs per SM behind a configuration's count
 template <typename T>
 int stress_ctas_per_sm();
 template <typename T>

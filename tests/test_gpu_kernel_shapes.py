@@ -25,3 +25,23 @@ def test_double_precision_stress_tiles(evp, shape, model, extra):
     ref = oracle.stress_rhs(st.U, st.V, st.W, st.B, g, prm)
     for c in range(6):
         assert rel(out[c].cpu().numpy(), ref[c]) < 1e-12, (c, rel(out[c].cpu().numpy(), ref[c]))
+
+
+# momentum tiles: 64 x 4 (nx a multiple of 64), 32 x 8, element-wise staging (nx % 4 = 2);
+# the last tile row holding one row, the wall rows in one tile, chunks with a remainder;
+# Newtonian states stage no stress
+@pytest.mark.parametrize("shape", [(64, 4, 8, True), (64, 5, 27, True), (128, 9, 8, True), (32, 8, 9, True),
+                                   (36, 17, 8, True), (18, 13, 16, True), (64, 18, 54, False), (54, 16, 8, False)])
+@pytest.mark.parametrize("model", ['oldroyd_b', 'newtonian'])
+@pytest.mark.parametrize("prec,tol", [(0, 1e-10), (1, 1e-5)])
+def test_momentum_tiles(evp, shape, model, prec, tol):
+    sim, st, g, prm = setup_case(evp, shape, model, {}, prec, dpdx=0.3)
+    # a quarter of the explicit viscous limit dt 4 mu_s sum 1/h^2 <= 2.51
+    h2 = sum((n / l) ** 2 for n, l in zip(shape[:3], (g.lx, g.ly, g.lz)))
+    dt = min(1e-3, 0.25 * 2.51 / (4 * 0.4 / 2.0 * h2))
+    for _ in range(2):
+        sim.step(dt)
+        st = oracle.rk3_step(st, dt, g, prm, force=(0.3, 0.0, 0.0))
+    sim.sync()
+    for f, ref in ((evp.EVP_U, st.U), (evp.EVP_V, st.V), (evp.EVP_W, st.W)):
+        assert rel(sim.get(f), ref) < tol, (f, rel(sim.get(f), ref))
