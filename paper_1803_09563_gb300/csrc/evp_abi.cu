@@ -366,18 +366,19 @@ int run_poisson(evp_state* s, const T* Us, const T* Vs, const T* Ws, const T* rh
 }
 
 // Implicit viscous option: field <- solution of x - c lap(x) = field for one
-// velocity component (kind_v: the v rule), in place through the spectral buffer
+// velocity component (kind_v: the v rule), in place through a spectral buffer and, with
+// walls, a scratch for the sweep
 template <typename T>
-int run_helmholtz(evp_state* s, T* field, double c, int k, bool kind_v) {
+PoissonArgs<T> helmholtz_args(evp_state* s, T* field, double c, int k, bool kind_v, void* spec, double* scratch) {
     PoissonArgs<T> a;
     a.Us = a.Vs = a.Ws = nullptr;
     a.rhs = field;
     a.rscale = T(1);
-    a.spec = static_cast<typename Cplx<T>::type*>(s->spec);
+    a.spec = static_cast<typename Cplx<T>::type*>(spec);
     a.psi = field;
     a.norm = poisson_norm<T>(s);
     a.out_scale = s->g.walls_y ? T(a.norm) : T(1);
-    a.scratch = s->thomas_d;
+    a.scratch = scratch;
     if (s->g.walls_y) {
         const double dy = s->g.ly / s->g.ny;
         a.ttab = s->helm[k][kind_v ? 1 : 0];
@@ -385,7 +386,34 @@ int run_helmholtz(evp_state* s, T* field, double c, int k, bool kind_v) {
     } else {
         a.hcoef = T(c);
     }
-    cudaError_t e = launch_poisson<T>(geo_of<T>(s), tables_of<T>(s), a, s->st, hook_of(s));
+    return a;
+}
+
+// The three components' solves.  With a stress all three go through each pass in one
+// launch (the batched passes): on grids of a million cells and less a pass of one
+// component leaves most SMs idle, and 96 x 100 x 72 spends 1.6 ms of two steps in 24
+// chains of five small launches, 1.2 ms in twelve.  The second and third spectral buffer
+// and scratch live in arrays that nothing reads between the momentum step and the next
+// stress update: the summed stress (two arrays for (nx + 2) ny nz elements) and B^{k-1}
+// (three arrays for as many doubles).  States without them solve one after the other.
+template <typename T>
+int run_helmholtz(evp_state* s, T* const (&star)[3], void* const (&b_old)[6], double c, int k) {
+    const Geo<T> g = geo_of<T>(s);
+    const FFTTables<T> tb = tables_of<T>(s);
+    const TimingHook th = hook_of(s);
+    cudaError_t e = cudaSuccess;
+    if (s->S[0]) {
+        PoissonBatch<T> p;
+        p.a[0] = helmholtz_args<T>(s, star[0], c, k, false, s->spec, s->thomas_d);
+        p.a[1] = helmholtz_args<T>(s, star[1], c, k, true, s->S[0], static_cast<double*>(b_old[0]));
+        p.a[2] = helmholtz_args<T>(s, star[2], c, k, false, s->S[2], static_cast<double*>(b_old[3]));
+        e = launch_poisson_batch<T>(g, tb, p, 3, sizeof(T) == 4 ? 16 : 8, s->st, th);
+    } else {
+        for (int q = 0; q < 3 && e == cudaSuccess; ++q) {
+            const PoissonArgs<T> a = helmholtz_args<T>(s, star[q], c, k, q == 1, s->spec, s->thomas_d);
+            e = launch_poisson<T>(g, tb, a, s->st, th);
+        }
+    }
     return e == cudaSuccess ? EVP_OK : cuda_fail(e, "helmholtz");
 }
 
@@ -524,9 +552,8 @@ int substep_t(evp_state* s, double dt, int k, bool last_in_step) {
     if (s->prm.viscous_implicit) {
         // Helmholtz solve per component: u* - alpha dt mu_s lap u* = rhs (Reading 18)
         const double c = al * dt * s->mc.mu_s;
-        T* star[3] = {static_cast<T*>(s->U[1 - cu]), static_cast<T*>(s->V[1 - cu]), static_cast<T*>(s->W[1 - cu])};
-        for (int q = 0; q < 3; ++q)
-            if (int r = run_helmholtz<T>(s, star[q], c, k, q == 1)) return r;
+        T* const star[3] = {static_cast<T*>(s->U[1 - cu]), static_cast<T*>(s->V[1 - cu]), static_cast<T*>(s->W[1 - cu])};
+        if (int r = run_helmholtz<T>(s, star, s->B[cb], c, k)) return r;
     }
     if (s->n_part > 0) {
         // discrete-forcing IBM of the rigid particles: u* -> u** (Eqs. IBM, CoVe2)

@@ -403,7 +403,8 @@ int step_direct(evp_batch* b) {
                 c.status = s->d_status;
             }
             const evp_state* s0 = b->m[gr.idx[0]].s;
-            cudaError_t e = launch_poisson_batch<T>(geo_of<T>(s0), tables_of<T>(s0), *pp, n, gr.tk, b->st);
+            cudaError_t e = launch_poisson_batch<T>(geo_of<T>(s0), tables_of<T>(s0), *pp, n, gr.tk, b->st,
+                                                        TimingHook{nullptr, nullptr, nullptr});
             if (e != cudaSuccess) return bcuda(e, "batched Poisson passes");
             e = launch_correct_batch<T>(geo_of<T>(s0), *cp, n, b->st);
             if (e != cudaSuccess) return bcuda(e, "batched correction");

@@ -641,7 +641,7 @@ int momentum_ctas_per_sm();
 // that share grid g and tables tb; tk: kx columns per block of the column passes
 template <typename T>
 cudaError_t launch_poisson_batch(const Geo<T>& g, const FFTTables<T>& tb, const PoissonBatch<T>& p, int n, int tk,
-                                 cudaStream_t st);
+                                 cudaStream_t st, const TimingHook& th);
 template <typename T>
 cudaError_t launch_correct_batch(const Geo<T>& g, const CorrectBatch<T>& p, int n, cudaStream_t st);
 

@@ -1064,7 +1064,7 @@ struct PassLaunch {
                    R... rest) const {
         if (pb) {
             set_smem<T>((const void*)kb, smem);
-            return launch_k(kb, dim3(grid.x, grid.y, nb), block, smem, st, false, g, tb, *pb, rest...);
+            return launch_k(kb, dim3(grid.x, grid.y, nb), block, smem, st, pdl, g, tb, *pb, rest...);
         }
         set_smem<T>((const void*)ks, smem);
         return launch_k(ks, grid, block, smem, st, pdl, g, tb, *a, rest...);
@@ -1203,12 +1203,11 @@ cudaError_t launch_poisson(const Geo<T>& g, const FFTTables<T>& tb, const Poisso
 
 template <typename T>
 cudaError_t launch_poisson_batch(const Geo<T>& g, const FFTTables<T>& tb, const PoissonBatch<T>& p, int n, int tk,
-                                 cudaStream_t st) {
+                                 cudaStream_t st, const TimingHook& th) {
     if (n <= 0) return cudaSuccess;
     if (n > EVP_BATCH_MAX) return cudaErrorInvalidValue;
-    const PassLaunch<T> L{nullptr, &p, n, st, false};
-    const TimingHook none{nullptr, nullptr, nullptr};
-    return poisson_chain<T>(g, tb, L, tk, none);
+    const PassLaunch<T> L{nullptr, &p, n, st, th.pdl};
+    return poisson_chain<T>(g, tb, L, tk, th);
 }
 
 template <typename T>
@@ -1252,9 +1251,11 @@ cudaError_t launch_correct_batch(const Geo<T>& g, const CorrectBatch<T>& p, int 
 }
 
 template cudaError_t launch_poisson_batch<float>(const Geo<float>&, const FFTTables<float>&,
-                                                 const PoissonBatch<float>&, int, int, cudaStream_t);
+                                                 const PoissonBatch<float>&, int, int, cudaStream_t,
+                                                 const TimingHook&);
 template cudaError_t launch_poisson_batch<double>(const Geo<double>&, const FFTTables<double>&,
-                                                  const PoissonBatch<double>&, int, int, cudaStream_t);
+                                                  const PoissonBatch<double>&, int, int, cudaStream_t,
+                                                  const TimingHook&);
 template cudaError_t launch_correct_batch<float>(const Geo<float>&, const CorrectBatch<float>&, int, cudaStream_t);
 template cudaError_t launch_correct_batch<double>(const Geo<double>&, const CorrectBatch<double>&, int,
                                                   cudaStream_t);
