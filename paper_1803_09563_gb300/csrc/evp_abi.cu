@@ -231,7 +231,7 @@ size_t plan(evp_state* s, char* base) {
     void* sol[3] = {nullptr, nullptr, nullptr};
     if (s->prm.penalization)
         for (int q = 0; q < 3; ++q) sol[q] = P(N * e);
-    void* mean = ab2 ? P(sizeof(double)) : nullptr;
+    void* mean = ab2 ? P(3 * sizeof(double)) : nullptr;
     void* mass = (ab2 && s->prm.ls_mass_iters > 0) ? P((2 * nparts + 2) * sizeof(double)) : nullptr;
     void* phs[3] = {nullptr, nullptr, nullptr};
     if (s->prm.soft_particles)
@@ -680,6 +680,7 @@ int ab2_step_t(evp_state* s, double dt) {
         I.eps = T(p.ls_eps_cells * dx);
         I.sigma = T(p.sigma);
         I.drho_g = T(p.rho_ratio > 0 ? 0.0 : p.drho_g);
+        I.rho_ratio = double(T(p.rho_ratio));
         if ((e = launch_interface<T>(g, I, s->st, th)) != cudaSuccess) return cuda_fail(e, "interface");
     }
     const bool first = s->nstep == 0;

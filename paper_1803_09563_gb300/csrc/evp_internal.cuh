@@ -282,8 +282,9 @@ struct IfaceArgs {
     T* n[3];           // unit normal at centres
     T* f[3];           // interface force at centres
     double* partials;  // per-block sums of 1 - H
-    double* mean_1mH;  // domain mean of 1 - H
+    double* mean_1mH;  // [3]: domain mean of 1 - H; T mean drho_g; T mean density
     T eps, sigma, drho_g;
+    double rho_ratio = 0.0;
 };
 
 // soft particles: RK3 update of the solid fraction, phi^k = phi^{k-1} + dt (zeta R
@@ -357,7 +358,7 @@ struct MomAB2Args {
     T mu_s1, mu_s2, mu_p1, mu_p2, inv_lam, L2, a_fene;
     // density contrast (rho_ratio > 0): rho = H + rho_ratio (1 - H), gravity along -y
     T rho_ratio, gravity;
-    const double* mean_1mH;   // domain mean of 1 - H (for the mean density)
+    const double* mean_1mH;   // as IfaceArgs (the mean density)
 };
 
 // Dong-Shen split projection (Eqs. poisson-LS, projection-LS)
