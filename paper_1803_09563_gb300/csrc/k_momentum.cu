@@ -865,17 +865,25 @@ MomentumTiles momentum_tiles<float>(int nx, int ny) {   // the batch's tiles
 template <>
 MomentumTiles momentum_tiles<double>(int nx, int ny) { return {(nx * ny + COL_NT - 1) / COL_NT, 1}; }
 
-// planes per CTA: about two waves of CTAs, chunks of 24 planes at most (longer ones leave
-// the last wave emptier than their shorter start saves: 256^3 in 267 us with 22 to 26
-// planes, 276 with 32; the channel 256 x 128 x 128 within 3 % from 6 to 16 planes), small
-// grids down to one plane
+// planes per CTA: as the stress kernel's rule, the CTAs of the busiest SM times (planes +
+// 1), with one CTA's worth for the first planes' way in.  Within 4 % of the best chunk of a
+// sweep on ten grids from 32^3 to 256^3 (64^3 13.2 us with 4 planes, 16.5 with one; 96^3 25
+// with 8, 27.5 with 3; 256 x 128 x 128 78 with 10)
 template <>
 int momentum_planes<float>(int nx, int ny, int nz) {
-    const int tiles = (nx * ny + MomTall::NT - 1) / MomTall::NT;
-    int chunks = (2 * 152 * MOM_CTAS + tiles - 1) / tiles;
-    chunks = chunks > nz ? nz : chunks;
-    chunks = chunks < (nz + 23) / 24 ? (nz + 23) / 24 : chunks;
-    return (nz + chunks - 1) / chunks;
+    const int tx = momentum_wide(nx) ? MomWide::TX : MomTall::TX, ty = momentum_wide(nx) ? MomWide::TY : MomTall::TY;
+    const int tiles = ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
+    int best = 1;
+    long long cost = -1;
+    for (int kz = 1; kz <= nz && kz <= 64; ++kz) {
+        const int rem = nz % kz, chunks = nz / kz + (4 * rem > kz ? 1 : 0);
+        const long long c = (long long)((tiles * chunks + 151) / 152 + 1) * (kz + 1);
+        if (cost < 0 || c <= cost) {
+            cost = c;
+            best = kz;
+        }
+    }
+    return best;
 }
 // the busiest SM's planes, a CTA's start costing about half a plane
 template <>

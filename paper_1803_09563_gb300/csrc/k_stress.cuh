@@ -686,14 +686,27 @@ StressShape stress_shape(int, int) { return {TX, TY}; }
 template <typename T>
 size_t stress_smem(int, int) { return sizeof(StressSmem<T>); }
 
-// z planes per CTA: about four waves of CTAs over all SMs (two CTAs per SM); small
-// grids go down to one plane per CTA so that every SM works
+// z planes per CTA.  An SM works through its CTAs' planes at one rate whether one or two
+// are resident, and a CTA's start (seven planes of its own columns and the halo of one)
+// costs about one plane more, so the time goes as the CTAs of the busiest SM, plus a
+// quarter for the first loads and the last CTA, times (planes + 1).  A last chunk of a
+// quarter's length or less rides along.  On eleven grids from 32^3 to 256^3 this picks the
+// fastest chunk of a sweep or one within 4 % of it, where a fixed four waves took
+// 64^3 28 us (22 now), 96^3 56 (49), 96 x 100 x 72 49 (44), 256 x 128 x 128 204 (199).
 template <typename T>
 int stress_planes(int nx, int ny, int nz) {
     const int tiles = ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
-    int chunks = (4 * 152 * 2 + tiles - 1) / tiles;
-    chunks = chunks > nz ? nz : chunks;
-    return (nz + chunks - 1) / chunks;
+    int best = 1;
+    double cost = -1.0;
+    for (int kz = 1; kz <= nz && kz <= 64; ++kz) {
+        const int rem = nz % kz, chunks = nz / kz + (4 * rem > kz ? 1 : 0);
+        const double c = (((tiles * chunks + 151) / 152) + 0.25) * (kz + 1);
+        if (cost < 0.0 || c < cost) {
+            cost = c;
+            best = kz;
+        }
+    }
+    return best;
 }
 
 template <typename T>
