@@ -399,7 +399,8 @@ typedef struct evp_batch_s evp_batch;
  * of the stress and momentum kernels, resident CTAs per SM of their persistent
  * grids (at most 2 and 4 in FP32, 1 and 2 in FP64), and kx columns per block of
  * the column FFT passes (4, 8 or 16; 16 only in FP32).  0 in a field: the
- * default (the heuristic of the single-state launches).                       */
+ * default (the heuristic of the single-state launches).  A batch of several FP32
+ * members sizes the work items of grids without an entry for the whole batch.  */
 typedef struct {
     int stress_kz, momentum_kz;
     int stress_ctas_per_sm, momentum_ctas_per_sm;

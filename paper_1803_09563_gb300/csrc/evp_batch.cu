@@ -99,13 +99,38 @@ bool complete_config(const evp_grid& g, int precision, evp_tile_config& c) {
            (c.fft_cols == 4 || c.fft_cols == 8 || (c.fft_cols == 16 && f32));
 }
 
-evp_tile_config lookup_config(const evp_grid& g, int precision, int model) {
+// the grid's entry in the table (tuned or set: returns true), else the default
+bool find_config(const evp_grid& g, int precision, int model, evp_tile_config* out) {
     {
         std::lock_guard<std::mutex> lock(g_cfg_mutex);
         auto it = g_cfg.find(cfg_key(g, precision, model));
-        if (it != g_cfg.end()) return it->second;
+        if (it != g_cfg.end()) {
+            *out = it->second;
+            return true;
+        }
     }
-    return default_config(g, precision);
+    *out = default_config(g, precision);
+    return false;
+}
+
+// Planes per work item for members that have no entry in the table: the single-state
+// rules (k_stress.cuh, k_momentum.cu) on the whole launch's items, so that the small grids
+// of a batch are not cut into one-plane items (each with the start of a chunk) for an SM
+// count that the batch fills many times over.  start: what an SM pays beside its items.
+int batch_planes(const std::vector<std::pair<int, int>>& tiles_nz, double start) {
+    int best = 1, most = 1;
+    for (const auto& t : tiles_nz) most = std::max(most, t.second);
+    double cost = -1.0;
+    for (int kz = 1; kz <= most && kz <= 64; ++kz) {
+        long long items = 0;
+        for (const auto& t : tiles_nz) items += (long long)t.first * ((t.second + kz - 1) / kz);
+        const double c = ((items + 151) / 152 + start) * (kz + 1);
+        if (cost < 0.0 || c <= cost) {
+            cost = c;
+            best = kz;
+        }
+    }
+    return best;
 }
 
 bool same_grid(const evp_grid& a, const evp_grid& b) {
@@ -124,6 +149,7 @@ struct evp_batch_s {
         evp_state* s;
         double dt;
         evp_tile_config cfg;
+        bool own_cfg;           // cfg comes from the table (or the tuner)
     };
     std::vector<Member> m;
     bool use_graph = true;
@@ -146,6 +172,11 @@ struct evp_batch_s {
     std::vector<Group> groups;
     int4* d_work = nullptr;
     size_t work_cap = 0;
+    // side streams: launches of one phase that do not depend on one another (the groups'
+    // Poisson chains, the models' stress updates) run beside the batch's stream
+    static constexpr int SIDE = 4;
+    cudaStream_t side[SIDE] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t fork = nullptr, join[SIDE] = {nullptr, nullptr, nullptr, nullptr};
     // replayed steps: one executable graph per signature (cu, cb, dt of every member)
     struct Graph {
         bool valid = false;
@@ -177,6 +208,19 @@ void add_work(std::vector<int4>& w, int gi, const evp_grid& g, int nbx, int nby,
             for (int bx = 0; bx < nbx; ++bx) w.push_back(make_int4(gi, bx, by, bz));
 }
 
+// The side streams and events of a batch, made when a phase first has more than one launch
+int make_side(evp_batch* b) {
+    if (b->fork) return EVP_OK;
+    int prio = 0;
+    BCK(cudaStreamGetPriority(b->st, &prio));
+    for (int q = 0; q < evp_batch_s::SIDE; ++q) {
+        if (!b->side[q]) BCK(cudaStreamCreateWithPriority(&b->side[q], cudaStreamNonBlocking, prio));
+        if (!b->join[q]) BCK(cudaEventCreateWithFlags(&b->join[q], cudaEventDisableTiming));
+    }
+    BCK(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+    return EVP_OK;
+}
+
 // Rebuild the launch plan after a membership change: configurations, groups and
 // the device work lists (the batch's stream is idle when this writes them).
 int prepare(evp_batch* b) {
@@ -186,8 +230,11 @@ int prepare(evp_batch* b) {
     b->stress.clear();
     b->momentum.clear();
     b->groups.clear();
-    for (auto& mb : b->m)
-        mb.cfg = b->has_override ? b->override_cfg : lookup_config(mb.s->g, b->precision, mb.s->model);
+    for (auto& mb : b->m) {
+        mb.own_cfg = true;
+        if (b->has_override) mb.cfg = b->override_cfg;
+        else mb.own_cfg = find_config(mb.s->g, b->precision, mb.s->model, &mb.cfg);
+    }
     for (int i = 0; i < (int)b->m.size(); ++i) {
         const evp_state* s = b->m[i].s;
         const bool v = has_vec(s);
@@ -220,35 +267,60 @@ int prepare(evp_batch* b) {
             b->groups.push_back(gr);
         }
     }
+    // the longest chains first (run_beside deals them to the streams in turn)
+    auto cells = [&](const evp_batch_s::Group& gr) { return gr.idx.size() * b->m[gr.idx[0]].s->N; };
+    std::stable_sort(b->groups.begin(), b->groups.end(),
+                     [&](const evp_batch_s::Group& x, const evp_batch_s::Group& y) { return cells(x) > cells(y); });
     std::vector<int4> work;
     const int sms = num_sms();
+    const bool f32 = b->precision == EVP_FP32;
+    auto stress_grid = [&](const evp_grid& g) {
+        const StressShape sh = shape_of(g, b->precision);
+        return std::make_pair((g.nx + sh.tw - 1) / sh.tw, (g.ny + sh.th - 1) / sh.th);
+    };
+    auto momentum_grid = [&](const evp_grid& g) {
+        const MomentumTiles t = f32 ? momentum_tiles<float>(g.nx, g.ny) : momentum_tiles<double>(g.nx, g.ny);
+        return std::make_pair(t.x, t.y);
+    };
+    // the single-precision rules are the ones measured for many tiles
+    auto plan_planes = [&](const std::vector<int>& idx, auto grid_of, double start, int evp_tile_config::*field) {
+        if (!f32 || idx.size() < 2) return;
+        std::vector<std::pair<int, int>> t;
+        for (int i : idx) {
+            const auto n = grid_of(b->m[i].s->g);
+            t.emplace_back(n.first * n.second, b->m[i].s->g.nz);
+        }
+        const int kz = batch_planes(t, start);
+        for (int i : idx)
+            if (!b->m[i].own_cfg) b->m[i].cfg.*field = std::min(kz, b->m[i].s->g.nz);
+    };
     for (auto& l : b->stress) {
+        plan_planes(l.idx, stress_grid, 0.25, &evp_tile_config::stress_kz);
         l.work_off = (int)work.size();
         int per_sm = 1;
         for (int gi = 0; gi < (int)l.idx.size(); ++gi) {
             const auto& mb = b->m[l.idx[gi]];
-            const StressShape sh = shape_of(mb.s->g, b->precision);
-            add_work(work, gi, mb.s->g, (mb.s->g.nx + sh.tw - 1) / sh.tw, (mb.s->g.ny + sh.th - 1) / sh.th,
-                     mb.cfg.stress_kz);
+            const auto n = stress_grid(mb.s->g);
+            add_work(work, gi, mb.s->g, n.first, n.second, mb.cfg.stress_kz);
             per_sm = std::max(per_sm, mb.cfg.stress_ctas_per_sm);
-            l.smem = std::max(l.smem, b->precision == EVP_FP32 ? stress_smem<float>(mb.s->g.nx, mb.s->g.ny)
-                                                               : stress_smem<double>(mb.s->g.nx, mb.s->g.ny));
+            l.smem = std::max(l.smem, f32 ? stress_smem<float>(mb.s->g.nx, mb.s->g.ny)
+                                          : stress_smem<double>(mb.s->g.nx, mb.s->g.ny));
         }
         l.nwork = (int)work.size() - l.work_off;
-        l.ctas = per_sm * sms * (b->precision == EVP_FP32 ? stress_cta_factor<float>() : stress_cta_factor<double>());
+        l.ctas = per_sm * sms * (f32 ? stress_cta_factor<float>() : stress_cta_factor<double>());
     }
     for (auto& l : b->momentum) {
+        plan_planes(l.idx, momentum_grid, 1.0, &evp_tile_config::momentum_kz);
         l.work_off = (int)work.size();
         int per_sm = 1;
         for (int gi = 0; gi < (int)l.idx.size(); ++gi) {
             const auto& mb = b->m[l.idx[gi]];
-            const MomentumTiles t = b->precision == EVP_FP32 ? momentum_tiles<float>(mb.s->g.nx, mb.s->g.ny)
-                                                             : momentum_tiles<double>(mb.s->g.nx, mb.s->g.ny);
-            add_work(work, gi, mb.s->g, t.x, t.y, mb.cfg.momentum_kz);
+            const auto n = momentum_grid(mb.s->g);
+            add_work(work, gi, mb.s->g, n.first, n.second, mb.cfg.momentum_kz);
             per_sm = std::max(per_sm, mb.cfg.momentum_ctas_per_sm);
         }
         l.nwork = (int)work.size() - l.work_off;
-        l.ctas = sms * (b->precision == EVP_FP32 ? momentum_resident<float>(per_sm) : momentum_resident<double>(per_sm));
+        l.ctas = sms * (f32 ? momentum_resident<float>(per_sm) : momentum_resident<double>(per_sm));
     }
     if (work.size() > b->work_cap) {
         if (b->d_work) cudaFree(b->d_work);
@@ -268,6 +340,8 @@ int prepare(evp_batch* b) {
         BCK(cudaMemcpyAsync(b->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, b->st));
         BCK(cudaStreamSynchronize(b->st));
     }
+    if (b->stress.size() > 1 || b->momentum.size() > 1 || b->groups.size() > 1)
+        if (int r = make_side(b)) return r;
     b->dirty = false;
     return EVP_OK;
 }
@@ -275,6 +349,30 @@ int prepare(evp_batch* b) {
 }  // namespace
 
 namespace {
+
+// n independent launches go(q, stream), q = 0 .. n-1: the first and every fifth on the
+// batch's stream, the others on the side streams, which start after what the batch's
+// stream holds and are waited for by what it gets next.  Five grid sizes' Poisson chains
+// are six launches each of a few CTAs an SM; in sequence they took half of a mixed
+// batch's step.
+template <typename F>
+int run_beside(evp_batch* b, int n, F go) {
+    const int used = std::min(n - 1, evp_batch_s::SIDE);
+    if (used > 0) {
+        BCK(cudaEventRecord(b->fork, b->st));
+        for (int q = 0; q < used; ++q) BCK(cudaStreamWaitEvent(b->side[q], b->fork, 0));
+    }
+    int r = EVP_OK;
+    for (int q = 0; q < n && r == EVP_OK; ++q) {
+        const int lane = q % (evp_batch_s::SIDE + 1);
+        r = go(q, lane == 0 ? b->st : b->side[lane - 1]);
+    }
+    for (int q = 0; q < used; ++q) {        // joined on an error too
+        BCK(cudaEventRecord(b->join[q], b->side[q]));
+        BCK(cudaStreamWaitEvent(b->st, b->join[q], 0));
+    }
+    return r;
+}
 
 // One RK3 step of every member with direct launches (also what a graph captures).
 template <typename T>
@@ -289,7 +387,8 @@ int step_direct(evp_batch* b) {
         const bool read_hist = xi != 0.0, write_hist = k != 2;
         const int mode = !read_hist ? 1 : (write_hist ? 2 : 3);
         // ---- S1 + S2: stress update (Eq. rk3tau), one persistent launch per (model, staging)
-        for (const auto& l : b->stress) {
+        int r = run_beside(b, (int)b->stress.size(), [&](int q, cudaStream_t st) -> int {
+            const auto& l = b->stress[q];
             for (int gi = 0; gi < (int)l.idx.size(); ++gi) {
                 const auto& mb = b->m[l.idx[gi]];
                 evp_state* s = mb.s;
@@ -322,11 +421,13 @@ int step_direct(evp_batch* b) {
                 a.mu_p1 = a.mu_p2 = T(0);
             }
             const cudaError_t e =
-                launch_stress_batch<T>(*sp, l.model, mode, l.vec, b->d_work + l.work_off, l.nwork, l.ctas, l.smem, b->st);
-            if (e != cudaSuccess) return bcuda(e, "batched stress kernel");
-        }
+                launch_stress_batch<T>(*sp, l.model, mode, l.vec, b->d_work + l.work_off, l.nwork, l.ctas, l.smem, st);
+            return e == cudaSuccess ? EVP_OK : bcuda(e, "batched stress kernel");
+        });
+        if (r) return r;
         // ---- S3: momentum predictor (Eq. rk3) with the summed stress
-        for (const auto& l : b->momentum) {
+        r = run_beside(b, (int)b->momentum.size(), [&](int q, cudaStream_t st) -> int {
+            const auto& l = b->momentum[q];
             for (int gi = 0; gi < (int)l.idx.size(); ++gi) {
                 const auto& mb = b->m[l.idx[gi]];
                 evp_state* s = mb.s;
@@ -366,11 +467,13 @@ int step_direct(evp_batch* b) {
                 a.cn = 0;
             }
             const cudaError_t e =
-                launch_momentum_batch<T>(*mp, l.vec, b->d_work + l.work_off, l.nwork, l.ctas, b->st);
-            if (e != cudaSuccess) return bcuda(e, "batched momentum kernel");
-        }
+                launch_momentum_batch<T>(*mp, l.vec, b->d_work + l.work_off, l.nwork, l.ctas, st);
+            return e == cudaSuccess ? EVP_OK : bcuda(e, "batched momentum kernel");
+        });
+        if (r) return r;
         // ---- S4 - S8: Poisson passes and correction per same-grid group
-        for (const auto& gr : b->groups) {
+        r = run_beside(b, (int)b->groups.size(), [&](int q, cudaStream_t st) -> int {
+            const auto& gr = b->groups[q];
             const int n = (int)gr.idx.size();
             for (int gi = 0; gi < n; ++gi) {
                 const auto& mb = b->m[gr.idx[gi]];
@@ -403,12 +506,13 @@ int step_direct(evp_batch* b) {
                 c.status = s->d_status;
             }
             const evp_state* s0 = b->m[gr.idx[0]].s;
-            cudaError_t e = launch_poisson_batch<T>(geo_of<T>(s0), tables_of<T>(s0), *pp, n, gr.tk, b->st,
-                                                        TimingHook{nullptr, nullptr, nullptr});
+            cudaError_t e = launch_poisson_batch<T>(geo_of<T>(s0), tables_of<T>(s0), *pp, n, gr.tk, st,
+                                                    TimingHook{nullptr, nullptr, nullptr});
             if (e != cudaSuccess) return bcuda(e, "batched Poisson passes");
-            e = launch_correct_batch<T>(geo_of<T>(s0), *cp, n, b->st);
-            if (e != cudaSuccess) return bcuda(e, "batched correction");
-        }
+            e = launch_correct_batch<T>(geo_of<T>(s0), *cp, n, st);
+            return e == cudaSuccess ? EVP_OK : bcuda(e, "batched correction");
+        });
+        if (r) return r;
         for (auto& mb : b->m) mb.s->cb = 1 - mb.s->cb;
     }
     return EVP_OK;
@@ -513,7 +617,7 @@ int evp_batch_admit(evp_batch* b, evp_state* s, double dt) {
         return bfail(EVP_ERR_OOM, "admitting the state would exceed the batch's memory budget");
     BCK(cudaStreamSynchronize(s->st));
     BCK(cudaStreamSynchronize(b->st));
-    b->m.push_back({s, dt, evp_tile_config{}});
+    b->m.push_back({s, dt, evp_tile_config{}, false});
     b->used += s->arena_bytes;
     s->batch = b;
     s->batch_st = b->st;
@@ -564,6 +668,11 @@ int evp_batch_destroy(evp_batch* b) {
     b->m.clear();
     drop_graphs(b);
     if (b->d_work) cudaFree(b->d_work);
+    for (int q = 0; q < evp_batch_s::SIDE; ++q) {
+        if (b->side[q]) cudaStreamDestroy(b->side[q]);
+        if (b->join[q]) cudaEventDestroy(b->join[q]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     if (b->own_stream) cudaStreamDestroy(b->st);
     delete b;
     return EVP_OK;
@@ -586,7 +695,7 @@ int evp_tile_config_set(const evp_grid* grid, int precision, evp_model model, co
 int evp_tile_config_get(const evp_grid* grid, int precision, evp_model model, evp_tile_config* out) {
     if (!grid || !out) return bfail(EVP_ERR_ARG, "null argument");
     if (precision != EVP_FP32 && precision != EVP_FP64) return bfail(EVP_ERR_ARG, "bad precision");
-    *out = lookup_config(*grid, precision, model);
+    find_config(*grid, precision, model, out);
     return EVP_OK;
 }
 
