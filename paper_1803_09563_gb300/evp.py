@@ -160,13 +160,14 @@ def _check(code):
     return code
 
 
-def _ptr(a):
-    """(pointer, on_device, nbytes) of a torch tensor or numpy array (contiguous)."""
+def _ptr(a, synchronize=True):
+    """(pointer, on_device, nbytes) of a torch tensor or numpy array (contiguous).
+    ``synchronize``: finish torch's pending work on a device tensor first."""
     try:
         import torch
         if isinstance(a, torch.Tensor):
             assert a.is_contiguous()
-            if a.is_cuda and not torch.cuda.is_current_stream_capturing():
+            if synchronize and a.is_cuda and not torch.cuda.is_current_stream_capturing():
                 # the library works on its own stream: finish torch's pending work on
                 # the tensor (a stream being captured orders the work by the capture
                 # and may not be synchronised)
@@ -230,7 +231,12 @@ def evp_get_field(state, field, dst):
 def _field_arrays(fields, bufs):
     if len(fields) != len(bufs):
         raise ValueError('one buffer per field')
-    ptrs = [_ptr(b) for b in bufs]
+    # torch's current stream is the same for every buffer of a device: wait for it once
+    seen, ptrs = set(), []
+    for b in bufs:
+        dev = getattr(b, 'device', None)
+        ptrs.append(_ptr(b, synchronize=dev not in seen))
+        seen.add(dev)
     devs = {d for _, d, _ in ptrs}
     if len(devs) > 1:
         raise ValueError('all buffers on the host or all on the device')

@@ -45,3 +45,26 @@ def test_momentum_tiles(evp, shape, model, prec, tol):
     sim.sync()
     for f, ref in ((evp.EVP_U, st.U), (evp.EVP_V, st.V), (evp.EVP_W, st.W)):
         assert rel(sim.get(f), ref) < tol, (f, rel(sim.get(f), ref))
+
+
+# several fields to device buffers in one launch: whole and broken 16-byte words, buffers
+# off the 16-byte grid, buffers that overlap (copied in order)
+@pytest.mark.parametrize("shape", [(8, 4, 8, True), (18, 5, 9, True), (64, 32, 24, False)])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_device_field_copies(evp, shape, prec):
+    import torch
+    sim, _, _, _ = setup_case(evp, shape, 'oldroyd_b', {}, prec)
+    n = sim.shape[0] * sim.shape[1] * sim.shape[2]
+    fields = [evp.EVP_U, evp.EVP_P, evp.EVP_BXY, evp.EVP_BZZ]
+    want = [sim.get(f).ravel() for f in fields]
+    for skew in (0, 1, 2):
+        pool = torch.full((4 * (n + 8),), float('nan'), dtype=sim.dtype, device='cuda')
+        bufs = [pool[q * (n + 8) + skew:q * (n + 8) + skew + n] for q in range(4)]
+        evp.evp_get_fields(sim.handle, fields, bufs)
+        for b, w in zip(bufs, want):
+            assert np.array_equal(b.cpu().numpy(), w)
+        assert int(torch.isnan(pool).sum()) == 32
+    pool = torch.zeros(2 * n, dtype=sim.dtype, device='cuda')
+    evp.evp_get_fields(sim.handle, fields[:2], [pool[:n], pool[n // 2:n // 2 + n]])
+    assert np.array_equal(pool[n // 2:n // 2 + n].cpu().numpy(), want[1])
+    assert np.array_equal(pool[:n // 2].cpu().numpy(), want[0][:n // 2])
