@@ -240,9 +240,9 @@ size_t plan(evp_state* s, char* base) {
     if (s->prm.viscous_implicit && g.walls_y)
         for (int k = 0; k < 3; ++k)
             for (int q = 0; q < 2; ++q) helm[k][q] = P((size_t)(g.nz / 2 + 1) * g.ny * nxh * sizeof(double2));
-    void* st = P(sizeof(unsigned));
+    void* st = P(2 * sizeof(unsigned));    // the status word; the residual's own for evp_diagnostics
     void* md = P(sizeof(unsigned long long));
-    void* dg = P((evp::DIAG_BLOCKS + 1) * sizeof(evp::DiagPart));
+    void* dg = P(evp::DIAG_BLOCKS * sizeof(evp::DiagPart) + sizeof(evp::DiagResult));
     if (base) {
         s->P = p; s->PSI = psi; s->spec = spec;
         s->twx = twx; s->twy = twy; s->twz = twz;
@@ -1434,13 +1434,21 @@ int evp_sync(evp_state* s, unsigned* bits, double* max_div) {
                                           (const double*)s->W[cu], ix, iy, iz, s->d_maxdiv, s->d_status, s->st);
         if (e != cudaSuccess) return cuda_fail(e, "divergence residual");
     }
+    // the status word and the residual lie next to one another in the arena: one copy and
+    // one wait (five of each cost more than the residual kernel)
+    unsigned char words[512];
+    const size_t span = reinterpret_cast<char*>(s->d_maxdiv) - reinterpret_cast<char*>(s->d_status);
+    if (span + sizeof(unsigned long long) > sizeof(words)) return fail(EVP_ERR_CUDA, "arena layout");
+    CK(cudaMemcpyAsync(words, s->d_status, span + sizeof(unsigned long long), cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
     unsigned st = 0;
     unsigned long long md = 0;
-    CK(cudaMemcpy(&st, s->d_status, sizeof(st), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(&md, s->d_maxdiv, sizeof(md), cudaMemcpyDeviceToHost));
-    CK(cudaMemsetAsync(s->d_status, 0, sizeof(unsigned), s->st));
-    CK(cudaStreamSynchronize(s->st));
+    std::memcpy(&st, words, sizeof(st));
+    std::memcpy(&md, words + span, sizeof(md));
+    if (st) {
+        CK(cudaMemsetAsync(s->d_status, 0, sizeof(unsigned), s->st));
+        CK(cudaStreamSynchronize(s->st));
+    }
     if (bits) *bits = st;
     if (max_div) {
         double d;
@@ -1463,7 +1471,7 @@ int evp_diagnostics(evp_state* s, evp_diag* out) {
     const int cu = s->cu, cb = s->cb;
     const double ix = s->g.nx / s->g.lx, iy = s->g.ny / s->g.ly, iz = s->g.nz / s->g.lz;
     DiagPart* parts = static_cast<DiagPart*>(s->diag);
-    DiagPart* res = parts + DIAG_BLOCKS;
+    DiagResult* res = reinterpret_cast<DiagResult*>(parts + DIAG_BLOCKS);
     auto go = [&](auto zero) -> int {
         using T = decltype(zero);
         DiagArgs<T> a;
@@ -1483,23 +1491,19 @@ int evp_diagnostics(evp_state* s, evp_diag* out) {
             a.H = static_cast<const T*>(s->HF);
             a.mp1 = (1.0 - s->prm.beta) * (1.0 / s->prm.Re);   // mu_p of fluid 1, as the AB2 step forms it
         }
+        // the residual raises its status bit in a word of its own, so that evp_sync reports
+        // only what the steps raised
         cudaError_t e = launch_div_residual<T>(geo_of<T>(s), a.U, a.V, a.W, ix, iy, iz, s->d_maxdiv,
-                                               s->d_status, s->st);
-        if (e == cudaSuccess) e = launch_diag<T>(geo_of<T>(s), a, parts, res, s->st);
+                                               s->d_status + 1, s->st);
+        if (e == cudaSuccess) e = launch_diag<T>(geo_of<T>(s), a, parts, s->d_maxdiv, res, s->st);
         return e == cudaSuccess ? EVP_OK : cuda_fail(e, "diagnostics kernels");
     };
-    // the residual kernel would OR EVP_BIT_NONFINITE into the status word: read the
-    // word first and put it back, so that evp_sync reports only what the steps raised
-    unsigned st_before = 0;
-    CK(cudaMemcpyAsync(&st_before, s->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, s->st));
     if (int r = s->fp32 ? go(float(0)) : go(double(0))) return r;
-    DiagPart h;
-    unsigned long long md = 0;
-    CK(cudaMemcpyAsync(&h, res, sizeof(h), cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(&md, s->d_maxdiv, sizeof(md), cudaMemcpyDeviceToHost, s->st));
+    DiagResult host;
+    CK(cudaMemcpyAsync(&host, res, sizeof(host), cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
-    CK(cudaMemcpyAsync(s->d_status, &st_before, sizeof(unsigned), cudaMemcpyHostToDevice, s->st));
-    CK(cudaStreamSynchronize(s->st));
+    const DiagPart& h = host.p;
+    const unsigned long long md = host.maxdiv;
     const double dv = s->g.lx / s->g.nx * (s->g.ly / s->g.ny) * (s->g.lz / s->g.nz);
     out->kinetic_energy = 0.5 * dv * h.ke;
     std::memcpy(&out->max_div, &md, sizeof(double));

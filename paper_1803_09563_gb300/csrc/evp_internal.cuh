@@ -667,6 +667,10 @@ struct DiagPart {
     unsigned long long yielded;    // cells with F > 0
     unsigned long long nonfinite;  // cells with a NaN or infinite value
 };
+struct DiagResult {                // what evp_diagnostics reads back
+    DiagPart p;
+    unsigned long long maxdiv;     // bits of the residual's double
+};
 template <typename T>
 struct DiagArgs {
     const T* U;
@@ -679,9 +683,11 @@ struct DiagArgs {
     double tau_y;
     int yield_mode;    // 0: no yield surface, 1: every cell flows, 2: Saramito |tau^d| > tau_y
 };
-// two launches on st: block partials into parts[0 .. DIAG_BLOCKS), their fold into *out
+// two launches on st: block partials into parts[0 .. DIAG_BLOCKS), their fold and *maxdiv
+// into *out
 template <typename T>
-cudaError_t launch_diag(const Geo<T>& g, const DiagArgs<T>& a, DiagPart* parts, DiagPart* out, cudaStream_t st);
+cudaError_t launch_diag(const Geo<T>& g, const DiagArgs<T>& a, DiagPart* parts, const unsigned long long* maxdiv,
+                        DiagResult* out, cudaStream_t st);
 
 template <typename T>
 cudaError_t launch_ls_stage(const Geo<T>& g, const LsArgs<T>& a, bool reinit, cudaStream_t st,

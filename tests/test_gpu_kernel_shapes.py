@@ -68,3 +68,36 @@ def test_device_field_copies(evp, shape, prec):
     evp.evp_get_fields(sim.handle, fields[:2], [pool[:n], pool[n // 2:n // 2 + n]])
     assert np.array_equal(pool[n // 2:n // 2 + n].cpu().numpy(), want[1])
     assert np.array_equal(pool[:n // 2].cpu().numpy(), want[0][:n // 2])
+
+
+# the single-precision monitoring filters where every cell is in doubt: a uniform B (all
+# determinants and traces equal), a deviator exactly at the yield stress, tiny and huge
+# values, an infinity; and a velocity at rest, uniform, and solenoidal to rounding
+@pytest.mark.parametrize("shape", [(36, 9, 8, True), (64, 16, 24, False)])
+@pytest.mark.parametrize("kind", ['uniform', 'yield', 'tiny', 'huge', 'inf'])
+def test_single_precision_monitoring_filters(evp, shape, kind):
+    from oracle import diagnostics as odg
+    sim, st, g, prm = setup_case(evp, shape, 'saramito', {'Bi': 0.4}, evp.EVP_FP32)
+    rng = np.random.default_rng(3)
+    full = lambda v: np.full(sim.shape, v)
+    B = {'uniform': lambda: [full(v) for v in (1.5, 0.25, 0.1, 1.2, 0.3, 1.1)],
+         # |tau^d| of a pure shear B = I + b e_xy is (mu_p/lambda) b: at the yield stress to rounding
+         'yield': lambda: [full(1.0), full(np.float32(0.4 / 2.0 * 0.8 / (0.6 / 2.0))), full(0.0), full(1.0), full(0.0), full(1.0)],
+         'tiny': lambda: [rng.uniform(0.5, 2.0, sim.shape) * 1e-20 for _ in range(6)],
+         'huge': lambda: [rng.uniform(0.5, 2.0, sim.shape) * 1e20 for _ in range(6)],
+         'inf': lambda: [b.copy() for b in st.B]}[kind]()
+    if kind == 'inf':
+        B[3][1, 2, 3] = np.inf
+    if kind in ('uniform', 'yield'):
+        U, V, W = full(0.0 if kind == 'uniform' else 0.75), full(0.0), full(0.0)
+    else:
+        U, V, W = st.U, st.V, st.W
+    sim.set_state(U, V, W, None, B)
+    rd = lambda a: np.asarray(a, dtype=np.float32).astype(np.float64)
+    with np.errstate(all='ignore'):
+        ref = odg.diagnostics(rd(U), rd(V), rd(W), [rd(b) for b in B], g, prm)
+    got = sim.diagnostics()
+    for f in ('min_det_B', 'max_tr_B', 'yielded_cells', 'nonfinite_cells'):
+        assert got[f] == ref[f], (f, got[f], ref[f])
+    assert got['kinetic_energy'] == pytest.approx(ref['kinetic_energy'], rel=1e-12, abs=0)
+    assert abs(got['max_div'] - ref['max_div']) <= 1e-12 * 2.0 / min(g.dx, g.dy, g.dz)
