@@ -101,3 +101,30 @@ def test_single_precision_monitoring_filters(evp, shape, kind):
         assert got[f] == ref[f], (f, got[f], ref[f])
     assert got['kinetic_energy'] == pytest.approx(ref['kinetic_energy'], rel=1e-12, abs=0)
     assert abs(got['max_div'] - ref['max_div']) <= 1e-12 * 2.0 / min(g.dx, g.dy, g.dz)
+
+
+# level-set stages whose z chunks hold three planes and a remainder: advection by u^n and
+# re-distancing of a field that repeats 32 times along z must repeat bit for bit, and be
+# what one period gives on its own (a grid of one plane per chunk)
+@pytest.mark.parametrize("nx,ny,walls", [(36, 113, True), (36, 128, False)])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_level_set_chunks(evp, nx, ny, walls, prec):
+    rng = np.random.default_rng(5)
+    one = (8, ny, nx)
+    k, j, i = np.meshgrid(*(np.arange(m) for m in one), indexing='ij')
+    phi = 0.2 * np.cos(2 * np.pi * i / nx) + 0.1 * np.cos(np.pi * j / ny) + 0.05 * np.sin(2 * np.pi * k / 8)
+    vel = [rng.uniform(-1, 1, one) for _ in range(3)]
+    if walls:
+        vel[1][:, -1] = 0.0
+    prm = evp.make_params(Re=35.0, Wi=1.0, beta=0.5, precision=prec, integrator=evp.EVP_AB2, mu_ratio=1.0,
+                          ls_eps_cells=1.5, sigma=0.1, drho_g=1.0, reinit_every=1, reinit_iters=2)
+    got = []
+    for reps in (1, 32):
+        sim = evp.Simulation(evp.make_grid(nx, ny, 8 * reps, 1.0, 4.0, 0.25 * reps, walls), 'oldroyd_b', prm)
+        sim.set_state(*(np.tile(v, (reps, 1, 1)) for v in vel))
+        sim.set(evp.EVP_PHI, np.tile(phi, (reps, 1, 1)))
+        sim.step(1e-3)
+        sim.sync()
+        got.append(sim.get(evp.EVP_PHI))
+    assert np.isfinite(got[0]).all() and not np.array_equal(got[0], phi.astype(got[0].dtype))
+    assert np.array_equal(got[1], np.tile(got[0], (32, 1, 1)))
