@@ -19,6 +19,7 @@
 // in shared memory.
 #include <algorithm>
 #include <cfloat>
+#include <climits>
 
 #include "evp_internal.cuh"
 #include "weno.cuh"
@@ -547,18 +548,22 @@ __device__ __forceinline__ void momentum_ab2_cell(const Geo<T>& g, const MomAB2A
     a.NH[2][c0] = Nz;
 }
 
-// z-marching tiles of the AB2 momentum step: a 32 x 4 tile walks a chunk of z
-// planes.  Planes k-1, k, k+1 of u, v, w, H and tau (built once per staged cell
+// z-marching tiles of the AB2 momentum step: a 32 x 4 tile walks a chunk of z planes.  Planes k-1, k, k+1 of u, v, w, H and tau (built once per staged cell
 // from B^n and H, instead of once per stencil use) and planes k, k+1 of the
 // interface force sit in shared memory with a one-cell halo in x and y, staged
 // with the periodic wraps and the wall ghost rules; the raw values of plane k+2
-// are loaded into registers before plane k is computed.
+// are loaded into registers before plane k is computed.  A staged cell's offset and its
+// wall ghost (the nearest row, u and w negated, v zero) are found once per thread.
+// Bound by instruction issue and shared-memory reads, about 45 a cell.  128 x 256 x 128 FP32:
+// 154 us with wraps and ghost rules at each of the 13 reads of a staged cell, 146 so
+// (32 x 8 tiles 150, 32 x 16 160).
 constexpr int AB_TX = 32, AB_TY = 4, AB_NT = AB_TX * AB_TY;
-constexpr int AB_W = AB_TX + 2, AB_H = AB_TY + 2, AB_PL = AB_W * AB_H;
+constexpr int AB_W = AB_TX + 2, AB_PL = AB_W * (AB_TY + 2);
 constexpr int AB_NE = (AB_PL + AB_NT - 1) / AB_NT;          // staged cells per thread
 
 template <typename T>
 struct Ab2Smem {
+    static constexpr int RES = sizeof(T) == 4 ? 4 : 3;      // CTAs per SM that the registers leave
     T U[3][AB_PL], V[3][AB_PL], W[3][AB_PL], H[3][AB_PL];    // ring slot = plane mod 3
     T TAU[6][3][AB_PL];
     T F[3][2][AB_PL];                                       // slot = plane mod 2
@@ -582,7 +587,8 @@ struct Ab2Src {
 };
 
 template <typename T, int MODEL>
-__global__ void __launch_bounds__(AB_NT) k_momentum_ab2(const Geo<T> g, const MomAB2Args<T> a, int kz_chunk) {
+__global__ void __launch_bounds__(AB_NT, Ab2Smem<T>::RES)
+k_momentum_ab2(const Geo<T> g, const MomAB2Args<T> a, int kz_chunk) {
     extern __shared__ __align__(16) unsigned char smraw[];
     Ab2Smem<T>& sm = *reinterpret_cast<Ab2Smem<T>*>(smraw);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * AB_TX + tx;
@@ -591,24 +597,33 @@ __global__ void __launch_bounds__(AB_NT) k_momentum_ab2(const Geo<T> g, const Mo
     const int i = i0 + tx, j = j0 + ty;
     const bool active = i < g.nx && j < g.ny;
     constexpr bool STRESS = MODEL != EVP_NEWTONIAN;
-    // raw values of one staged plane for this thread's cells
+    const size_t plane = (size_t)g.nx * g.ny;
+    // raw values of one staged plane for this thread's cells, their offsets in a plane
     T ru[AB_NE], rv[AB_NE], rw[AB_NE], rH[AB_NE], rB[6][AB_NE], rf[3][AB_NE];
+    int off[AB_NE];
+    bool ghost[AB_NE];
+#pragma unroll
+    for (int r = 0; r < AB_NE; ++r) {
+        const int e = min(tid + r * AB_NT, AB_PL - 1), ly = e / AB_W, lx = e - ly * AB_W;
+        // the halo of a ragged tile may reach past the ghosts: any cell does there
+        const int gi = min(i0 - 1 + lx, g.nx), gj = min(j0 - 1 + ly, g.ny);
+        off[r] = ycen(g, gj) * g.nx + wrap(gi, g.nx);
+        ghost[r] = g.walls && (gj < 0 || gj >= g.ny);
+    }
     auto load = [&](int q) {
+        const size_t o = (size_t)wrap(q, g.nz) * plane;
 #pragma unroll
         for (int r = 0; r < AB_NE; ++r) {
-            const int e = tid + r * AB_NT;
-            if (e >= AB_PL) continue;
-            const int ly = e / AB_W, lx = e - ly * AB_W;
-            // the halo of a ragged tile may reach past one period of a short x
-            const int gi = ((i0 - 1 + lx) % g.nx + g.nx) % g.nx, gj = j0 - 1 + ly;
-            ru[r] = ld_uw(g, a.U, gi, gj, q);
-            rv[r] = ld_v(g, a.V, gi, gj, q);
-            rw[r] = ld_uw(g, a.W, gi, gj, q);
-            rH[r] = ld_c(g, a.H, gi, gj, q);
+            if (tid + r * AB_NT >= AB_PL) continue;
+            const int c0 = off[r];
+            ru[r] = __ldg(a.U + o + c0);
+            rv[r] = __ldg(a.V + o + c0);
+            rw[r] = __ldg(a.W + o + c0);
+            rH[r] = __ldg(a.H + o + c0);
 #pragma unroll
-            for (int c = 0; c < 6; ++c) rB[c][r] = STRESS ? ld_c(g, a.B[c], gi, gj, q) : T(0);
+            for (int c = 0; c < 6; ++c) rB[c][r] = STRESS ? __ldg(a.B[c] + o + c0) : T(0);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) rf[c][r] = ld_c(g, a.f[c], gi, gj, q);
+            for (int c = 0; c < 3; ++c) rf[c][r] = __ldg(a.f[c] + o + c0);
         }
     };
     auto store = [&](int q) {
@@ -617,9 +632,9 @@ __global__ void __launch_bounds__(AB_NT) k_momentum_ab2(const Geo<T> g, const Mo
         for (int r = 0; r < AB_NE; ++r) {
             const int e = tid + r * AB_NT;
             if (e >= AB_PL) continue;
-            sm.U[s3][e] = ru[r];
-            sm.V[s3][e] = rv[r];
-            sm.W[s3][e] = rw[r];
+            sm.U[s3][e] = ghost[r] ? -ru[r] : ru[r];
+            sm.V[s3][e] = ghost[r] ? T(0) : rv[r];
+            sm.W[s3][e] = ghost[r] ? -rw[r] : rw[r];
             sm.H[s3][e] = rH[r];
             if (STRESS) {
                 T b[6];
@@ -826,13 +841,20 @@ cudaError_t launch_mass_correct(const Geo<T>& g, const MassArgs<T>& a, int mode,
 template <typename T>
 cudaError_t launch_momentum_ab2(const Geo<T>& g, int model, const MomAB2Args<T>& a, cudaStream_t st,
                                 const TimingHook& th) {
-    // z chunks: about four waves of four CTAs per SM; small grids down to one plane
-    const int tiles = ((g.nx + AB_TX - 1) / AB_TX) * ((g.ny + AB_TY - 1) / AB_TY);
-    int chunks = (4 * 152 * 4 + tiles - 1) / tiles;
-    chunks = chunks > g.nz ? g.nz : chunks;
-    const int kz = (g.nz + chunks - 1) / chunks;
-    chunks = (g.nz + kz - 1) / kz;
-    const dim3 block(AB_TX, AB_TY, 1), grid((g.nx + AB_TX - 1) / AB_TX, (g.ny + AB_TY - 1) / AB_TY, chunks);
+    // planes per chunk: the least (waves of CTAs) x (planes + 2), two planes being what a
+    // chunk's start costs
+    const int gx = (g.nx + AB_TX - 1) / AB_TX, gy = (g.ny + AB_TY - 1) / AB_TY;
+    int kz = 1;
+    long long best = LLONG_MAX;
+    for (int c = 1; c <= g.nz; ++c) {
+        const long long ctas = (long long)gx * gy * ((g.nz + c - 1) / c), slots = 152 * Ab2Smem<T>::RES;
+        const long long cost = (ctas + slots - 1) / slots * (c + 2);
+        if (cost < best) {
+            best = cost;
+            kz = c;
+        }
+    }
+    const dim3 block(AB_TX, AB_TY, 1), grid(gx, gy, (g.nz + kz - 1) / kz);
     const size_t smem = sizeof(Ab2Smem<T>);
     auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
