@@ -1041,7 +1041,10 @@ k_div_residual(const Geo<T> g, const T* __restrict__ U, const T* __restrict__ V,
                 if (lo > 0.f && lo < FLT_MAX) atomicMax(&top, __float_as_int(lo));
             }
             const double w0 = wide(wh), wm = wide(wb), vm = wide(vl);
-            const double dv = (wide(uh) - wide(ul)) * idx_d + (wide(vh) - vm) * idy_d + (w0 - wm) * idz_d;
+            // contraction written out: on a velocity that is solenoidal to rounding the order of
+            // the roundings is a few per cent of the residual
+            const double dx = __dsub_rn(wide(uh), wide(ul)), dy = __dsub_rn(wide(vh), vm), dz = __dsub_rn(w0, wm);
+            const double dv = __fma_rn(dz, idz_d, __fma_rn(dx, idx_d, __dmul_rn(dy, idy_d)));
             const unsigned long long ab = (unsigned long long)__double_as_longlong(dv) & 0x7fffffffffffffffull;
             // |dv| finite <=> its exponent field is not all ones
             if (ab >= 0x7ff0000000000000ull) bits |= EVP_BIT_NONFINITE;

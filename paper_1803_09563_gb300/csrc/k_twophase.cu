@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256, 3) k_ls_stage(const Geo<T> g, const LsArg
                 T dl, dr;              // left- and right-biased derivatives
                 if constexpr (sizeof(T) == 4) {
                     auto lr = [&](int m) { return make_float2(d[q][m], d[q][5 - m]); };
-                    const float2 r = weno5x2(lr(0), lr(1), lr(2), lr(3), lr(4), splat2(ih[q]));
+                    const float2 r = weno5x2<true>(lr(0), lr(1), lr(2), lr(3), lr(4), splat2(ih[q]));
                     dl = r.x;
                     dr = r.y;
                 } else {
@@ -125,13 +125,17 @@ __global__ void __launch_bounds__(256, 3) k_ls_stage(const Geo<T> g, const LsArg
                 // Godunov: (max(dl, 0), min(dr, 0)) for S > 0, (min(dl, 0), max(dr, 0)) else
                 const bool up = sg > T(0);
                 const T l = up ? dl : -dl, r = up ? -dr : dr;
-                sum += sqr(fmax(fmax(l, r), T(0)));
+                // the square rounded on its own
+                const T gr = fmax(fmax(l, r), T(0));
+                if constexpr (sizeof(T) == 4) sum = __fadd_rn(sum, __fmul_rn(gr, gr));
+                else sum = __dadd_rn(sum, __dmul_rn(gr, gr));
             }
             rhs = -sg * (sqrt(sum) - T(1));
         }
         // plain load: the third stage writes phi in place (each cell by its own thread)
         const T pn = a.pt_a != T(0) ? a.phin[o + col] : T(0);
-        a.out[o + col] = a.pt_a * pn + a.pt_b * (pc + a.dt * rhs);
+        const T x = fma(a.dt, rhs, pc);
+        a.out[o + col] = fma(a.pt_a, pn, a.pt_b * x);
     }
 }
 

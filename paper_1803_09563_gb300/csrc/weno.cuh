@@ -68,10 +68,14 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(rcp_approx(a.x), rcp_approx(a.y)); }
 
 // weno5<float> on two independent stencils at once (the lanes of each argument),
-// with the same operations in the same order.
+// with the same operations in the same order; which product of q1 is rounded on its own
+// is the compiler's choice in weno5<float>: v2's in the level-set stages (V1_FUSED), v1's
+// here otherwise.
+template <bool V1_FUSED = false>
 __device__ __forceinline__ float2 weno5x2(float2 v1, float2 v2, float2 v3, float2 v4, float2 v5, float2 scale) {
     const float2 eps = splat2(float(1.0e-6 * 12.0 / 13.0)), r = splat2(float(3.0 / 13.0));
-    const float2 q1 = fma2(v3, splat2(float(11.0 / 6.0)), fma2(v2, splat2(float(-7.0 / 6.0)), mul2(v1, splat2(float(1.0 / 3.0)))));
+    const float2 t = splat2(float(1.0 / 3.0)), s6 = splat2(float(-7.0 / 6.0));
+    const float2 q1 = fma2(v3, splat2(float(11.0 / 6.0)), V1_FUSED ? fma2(v1, t, mul2(v2, s6)) : fma2(v2, s6, mul2(v1, t)));
     const float2 q2 = fma2(v4, splat2(2.0f), fma2(v3, splat2(5.0f), neg2(v2)));
     const float2 q3 = fma2(v5, splat2(-0.5f), fma2(v4, splat2(2.5f), v3));
     const float2 e12 = sub2(v1, v2), e23 = sub2(v2, v3), e34 = sub2(v3, v4), e45 = sub2(v4, v5);
