@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(256, 3) k_ls_stage(const Geo<T> g, const LsArg
             }
         } else {
             const T f0 = __ldg(a.phi0 + o + col);
-            const T sg = f0 / sqrt(f0 * f0 + a.h * a.h);
+            const T sg = f0 / sqrt(fma(a.h, a.h, f0 * f0));
             const T ih[3] = {g.idx, g.idy, g.idz};
             T sum = T(0);
 #pragma unroll
