@@ -103,8 +103,27 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Shared memory of a tw x th tile, in doubles: two planes of B with a 3-cell halo;
 // second differences along x (columns -2 .. tw+1) and y (rows -2 .. th+1) and smooth_a
 // at the half points between them
-__host__ __device__ inline int tile_doubles(int tw, int th) {
+__host__ __device__ constexpr int tile_doubles(int tw, int th) {
     return 12 * (tw + 6) * (th + 6) + 12 * (tw + 4) * th + 12 * tw * (th + 4);
+}
+// The tiles that stress_shape chooses from: TW_MIN .. TW_MAX columns and the rows that
+// NT threads hold.  The largest one's bytes are the kernels' limit of dynamic shared
+// memory: the limit belongs to a kernel, not to a launch, and host threads with states on
+// different grids launch the same kernel, so a limit set to each launch's own size could
+// be lowered by another thread before the launch.
+constexpr int TW_MIN = 8, TW_MAX = 64;
+constexpr int largest_tile_bytes() {
+    int most = 0;
+    for (int tw = TW_MIN; tw <= TW_MAX; ++tw) {
+        const int d = tile_doubles(tw, NT / tw);
+        most = d > most ? d : most;
+    }
+    return most * (int)sizeof(double);
+}
+static_assert(2 * (largest_tile_bytes() + 1024) <= 228 * 1024, "two CTAs on an SM");
+template <typename K>
+cudaError_t raise_smem_limit(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, largest_tile_bytes());
 }
 
 // MODE: 0 = right-hand side only, 1 = update without history read, 2 = update reading
@@ -496,7 +515,7 @@ template <>
 StressShape stress_shape<double>(int nx, int ny) {
     StressShape best{32, 4};
     long long cost = -1;
-    for (int tw = 8; tw <= 64; ++tw) {
+    for (int tw = TW_MIN; tw <= TW_MAX; ++tw) {
         int th = NT / tw;
         th = th > ny ? ny : th;
         const long long c = (long long)((nx + tw - 1) / tw) * ((ny + th - 1) / th) * plane_cost(tw, th);
@@ -544,7 +563,7 @@ cudaError_t launch_stress<double>(const Geo<double>& g, const ModelConst& mc, co
     const dim3 grid((g.nx + s.tw - 1) / s.tw, (g.ny + s.th - 1) / s.th, (g.nz + kz - 1) / kz), block(NT);
     const size_t smem = (size_t)tile_doubles(s.tw, s.th) * sizeof(double);
     auto go = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (cudaError_t e = raise_smem_limit(kern)) return e;
         return launch_k(kern, grid, block, smem, st, th.pdl, g, mc, a, s.tw, s.th, kz);
     };
     const int mode = a.rhs_only ? 0 : (!a.read_hist ? 1 : (a.write_hist ? 2 : 3));
@@ -575,7 +594,7 @@ cudaError_t launch_stress_batch<double>(const StressBatch<double>& p, int model,
     if (nwork <= 0) return cudaSuccess;
     const dim3 grid(ctas < nwork ? ctas : nwork), block(NT);
     auto go = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (cudaError_t e = raise_smem_limit(kern)) return e;
         return launch_k(kern, grid, block, smem, st, false, p, work, nwork);
     };
     switch (model * 4 + mode) {

@@ -1,0 +1,54 @@
+"""Host threads that each use a state of their own: what one thread's launches set on a
+kernel must not reach another thread's launches."""
+
+import threading
+
+import numpy as np
+import pytest
+
+from test_gpu_parity import setup_case
+
+pytestmark = pytest.mark.gpu
+
+
+def in_threads(jobs):
+    """Run every job in a thread of its own, all started together; their exceptions."""
+    errors, gate = [], threading.Barrier(len(jobs))
+
+    def run(job):
+        try:
+            gate.wait()
+            job()
+        except Exception as e:
+            errors.append(e)
+    threads = [threading.Thread(target=run, args=(j,)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    return errors
+
+
+# grids whose double-precision stress tiles differ in shape and so in shared memory:
+# 32 x 4, 18 x 7 and 64 x 2 columns
+@pytest.mark.parametrize("model,extra", [('oldroyd_b', {}), ('saramito', {'Bi': 0.4})])
+def test_double_precision_stress_from_several_threads(evp, model, extra):
+    import torch
+    sims = [setup_case(evp, s, model, extra, evp.EVP_FP64)[0] for s in
+            ((32, 32, 8, False), (72, 54, 8, False), (128, 6, 8, True))]
+    outs = [torch.empty((6,) + s.shape, dtype=torch.float64, device='cuda') for s in sims]
+    want = []
+    for s, o in zip(sims, outs):
+        evp.evp_stress_rhs(s.handle, o)
+        s.sync()
+        want.append(o.cpu().numpy())
+
+    def job(s, o):
+        def repeat():
+            for _ in range(1500):
+                evp.evp_stress_rhs(s.handle, o)
+            s.sync()
+        return repeat
+    assert not in_threads([job(s, o) for s, o in zip(sims, outs)])
+    for w, o in zip(want, outs):
+        assert np.array_equal(w, o.cpu().numpy())
