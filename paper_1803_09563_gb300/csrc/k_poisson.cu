@@ -1085,9 +1085,16 @@ k_div_residual(const Geo<T> g, const T* __restrict__ U, const T* __restrict__ V,
 template <typename T>
 size_t col_smem(int n, int tk) { return 2 * (size_t)n * tk * sizeof(C<T>); }
 
-template <typename T>
-void set_smem(const void* f, size_t bytes) {
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// The limit of dynamic shared memory belongs to a kernel, not to a launch, and host
+// threads with states on different grids launch the same kernel: beyond the default the
+// limit is always set to what the largest pass takes (two buffers of 512 points of 16
+// single- or 8 double-precision columns), never to a launch's own size, which another
+// thread's launch may exceed.
+constexpr size_t SMEM_LIMIT = 2 * 512 * 128;
+cudaError_t set_smem(const void* f, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    if (bytes > SMEM_LIMIT) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT);
 }
 
 // Launch of one pass, single or batched.  Single: the state's arguments by value,
@@ -1105,10 +1112,10 @@ struct PassLaunch {
     cudaError_t go(KS ks, KB kb, dim3 grid, dim3 block, size_t smem, const Geo<T>& g, const FFTTables<T>& tb,
                    R... rest) const {
         if (pb) {
-            set_smem<T>((const void*)kb, smem);
+            if (cudaError_t e = set_smem((const void*)kb, smem)) return e;
             return launch_k(kb, dim3(grid.x, grid.y, nb), block, smem, st, pdl, g, tb, *pb, rest...);
         }
-        set_smem<T>((const void*)ks, smem);
+        if (cudaError_t e = set_smem((const void*)ks, smem)) return e;
         return launch_k(ks, grid, block, smem, st, pdl, g, tb, *a, rest...);
     }
 };

@@ -52,3 +52,29 @@ def test_double_precision_stress_from_several_threads(evp, model, extra):
     assert not in_threads([job(s, o) for s, o in zip(sims, outs)])
     for w, o in zip(want, outs):
         assert np.array_equal(w, o.cpu().numpy())
+
+
+# lines of 216, 384 and 512 points, whose column passes differ in shared memory beyond the
+# default limit
+@pytest.mark.parametrize("prec", [0, 1])
+def test_poisson_solves_from_several_threads(evp, prec):
+    import torch
+    sims = [setup_case(evp, (8, 8, nz, False), 'newtonian', {}, prec)[0] for nz in (216, 384, 512)]
+    rhs, psi, want = [], [], []
+    for s in sims:
+        r = torch.randn(s.shape, dtype=s.dtype, device='cuda', generator=torch.Generator('cuda').manual_seed(1))
+        rhs.append(r - r.mean())
+        psi.append(torch.empty_like(r))
+        evp.evp_poisson_solve(s.handle, rhs[-1], psi[-1])
+        s.sync()
+        want.append(psi[-1].cpu().numpy())
+
+    def job(s, r, p):
+        def repeat():
+            for _ in range(600):
+                evp.evp_poisson_solve(s.handle, r, p)
+            s.sync()
+        return repeat
+    assert not in_threads([job(*a) for a in zip(sims, rhs, psi)])
+    for w, p in zip(want, psi):
+        assert np.array_equal(w, p.cpu().numpy())
