@@ -307,8 +307,13 @@ int upload_tables(evp_state* s) {
         for (int m = 0; m < cnt; ++m) v[m] = (2.0 - 2.0 * std::cos(twopi * m / n)) / (h * h);
         return v;
     };
+    // the host tables stay until the stream has been waited for: a copy from pageable
+    // memory may still be reading it when cudaMemcpyAsync returns
+    std::vector<std::vector<T>> host;
+    host.reserve(8);
     auto put = [&](void* dst, const std::vector<double>& v) -> cudaError_t {
-        std::vector<T> t = to_t<T>(v);
+        host.push_back(to_t<T>(v));
+        const std::vector<T>& t = host.back();
         return cudaMemcpyAsync(dst, t.data(), t.size() * sizeof(T), cudaMemcpyHostToDevice, s->st);
     };
     CK(put(s->twx, tw(g.nx)));
@@ -331,12 +336,14 @@ int upload_tables(evp_state* s) {
         for (int q = 0; q < g.nz; ++q) t.push_back(std::cos(k * (q + 0.5) * dz));
         CK(put(s->trig, t));
     }
+    std::vector<double> M;
+    std::vector<float> F;
     if (g.walls_y) {
         // Thomas table (m_j, c'_j) per (kz <= nz/2, kx), built in FP64
-        const std::vector<double> M = thomas_table(g.ny, g.nz, nxh, dy, lx, lam(g.nz, g.nz / 2 + 1, dz));
+        M = thomas_table(g.ny, g.nz, nxh, dy, lx, lam(g.nz, g.nz / 2 + 1, dz));
         if (sizeof(T) == 4 && !s->prm.thomas_fp64) {
             // single-precision states sweep in double-single arithmetic (k_thomas)
-            const std::vector<float> F = thomas_table_ds(M);
+            F = thomas_table_ds(M);
             CK(cudaMemcpyAsync(s->thomas_m, F.data(), F.size() * sizeof(float), cudaMemcpyHostToDevice, s->st));
         } else {
             CK(cudaMemcpyAsync(s->thomas_m, M.data(), M.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
@@ -433,16 +440,21 @@ int prepare_helmholtz(evp_state* s, double dt) {
     static const double RK3_ALPHA_H[3] = {4.0 / 15.0, 1.0 / 15.0, 1.0 / 6.0};
     // on the state's stream: a copy on the legacy stream may still be on its way to the
     // device when cudaMemcpy returns (pageable memory is only staged by then), and a
-    // non-blocking stream does not wait for it
+    // non-blocking stream does not wait for it.  The host tables stay until the stream has
+    // been waited for: cudaMemcpyAsync may return before it has read pageable memory.
     CK(cudaStreamSynchronize(s->st));
+    std::vector<double> M[3][2];
+    std::vector<float> F[3][2];
     for (int k = 0; k < 3; ++k)
         for (int q = 0; q < 2; ++q) {
-            const std::vector<double> M = helmholtz_table(g.ny, g.nz, nxh, dy, lx, lz, RK3_ALPHA_H[k] * dt * mu_s, q == 1);
+            std::vector<double>& m = M[k][q];
+            std::vector<float>& f = F[k][q];
+            m = helmholtz_table(g.ny, g.nz, nxh, dy, lx, lz, RK3_ALPHA_H[k] * dt * mu_s, q == 1);
             if (s->fp32 && !s->prm.thomas_fp64) {
-                const std::vector<float> F = thomas_table_ds(M);
-                CK(cudaMemcpyAsync(s->helm[k][q], F.data(), F.size() * sizeof(float), cudaMemcpyHostToDevice, s->st));
+                f = thomas_table_ds(m);
+                CK(cudaMemcpyAsync(s->helm[k][q], f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice, s->st));
             } else {
-                CK(cudaMemcpyAsync(s->helm[k][q], M.data(), M.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
+                CK(cudaMemcpyAsync(s->helm[k][q], m.data(), m.size() * sizeof(double), cudaMemcpyHostToDevice, s->st));
             }
         }
     CK(cudaStreamSynchronize(s->st));

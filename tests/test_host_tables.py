@@ -170,3 +170,90 @@ def test_double_single_table_reproduces_the_doubles(tables):
     # the pinned system's row 0 (m = 1, c' = 0) and every system's last c' (0) are exact
     assert F[0, 0, 0, 0] == 1.0 and F[0, 0, 0, 1] == 0.0
     assert np.all(F[:, -1, :, 2] == 0.0) and np.all(F[:, -1, :, 3] == 0.0)
+
+
+UPLOADS = r'''
+#include <cuda_runtime.h>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <vector>
+// copies to the device that read their source as late as they are allowed to: when the
+// stream is waited for
+struct Copy { void* dst; const void* src; size_t n; };
+static std::vector<Copy> pending;
+static cudaError_t late_copy(void* dst, const void* src, size_t n, cudaMemcpyKind, cudaStream_t) {
+    pending.push_back({dst, src, n});
+    return cudaSuccess;
+}
+static cudaError_t late_sync(cudaStream_t) {
+    for (const Copy& c : pending) std::memcpy(c.dst, c.src, c.n);
+    pending.clear();
+    return cudaSuccess;
+}
+#define cudaMemcpyAsync late_copy
+#define cudaStreamSynchronize late_sync
+#include "evp_abi.cu"
+template <typename T>
+static int check(bool fp32) {
+    evp_state_s* s = new evp_state_s{};
+    s->g.nx = 24; s->g.ny = 40; s->g.nz = 36;
+    s->g.lx = 2.0; s->g.ly = 3.0; s->g.lz = 1.5;
+    s->g.walls_y = 1;
+    s->prm.Re = 2.0; s->prm.beta = 0.4; s->prm.Wi = 1.0; s->prm.viscous_implicit = 1;
+    s->prm.precision = fp32 ? EVP_FP32 : EVP_FP64;
+    s->model = EVP_OLDROYD_B;
+    s->fp32 = fp32;
+    s->elt = sizeof(T);
+    s->N = (size_t)24 * 40 * 36;
+    s->nxh = 13;
+    s->arena_bytes = plan(s, nullptr);
+    s->arena = static_cast<char*>(std::aligned_alloc(256, (s->arena_bytes + 255) / 256 * 256));
+    plan(s, s->arena);
+    if (upload_tables<T>(s) != EVP_OK) return 1;
+    for (double dt : {1e-2, 3e-3})
+        if (prepare_helmholtz(s, dt) != EVP_OK) return 2;
+    // what the tables hold against the tables themselves
+    const double dx = 2.0 / 24, dy = 3.0 / 40, dz = 1.5 / 36;
+    std::vector<double> lx(13), lz(19);
+    for (int m = 0; m < 13; ++m) lx[m] = (2.0 - 2.0 * std::cos(2.0 * M_PI * m / 24)) / (dx * dx);
+    for (int m = 0; m < 19; ++m) lz[m] = (2.0 - 2.0 * std::cos(2.0 * M_PI * m / 36)) / (dz * dz);
+    auto same = [&](const void* dev, const std::vector<double>& want) {
+        if (!fp32) return std::memcmp(dev, want.data(), want.size() * sizeof(double)) == 0;
+        const std::vector<float> f = thomas_table_ds(want);
+        return std::memcmp(dev, f.data(), f.size() * sizeof(float)) == 0;
+    };
+    const double al[3] = {4.0 / 15.0, 1.0 / 15.0, 1.0 / 6.0};
+    for (int k = 0; k < 3; ++k)
+        for (int q = 0; q < 2; ++q)
+            if (!same(s->helm[k][q], helmholtz_table(40, 36, 13, dy, lx, lz, al[k] * 3e-3 * 0.2, q == 1))) return 3;
+    if (!same(s->thomas_m, thomas_table(40, 36, 13, dy, lx, lz))) return 4;
+    const T* tw = static_cast<const T*>(s->twx);
+    for (int m = 0; m < 24; ++m)
+        if (std::fabs(tw[2 * m] - std::cos(2.0 * M_PI * m / 24)) > 1e-6) return 5;
+    return 0;
+}
+int main() {
+    const int a = check<double>(false), b = check<float>(true);
+    std::printf("%d %d\n", a, b);
+    return a || b;
+}
+'''
+
+
+def test_tables_outlive_their_uploads(tmp_path):
+    """The host side of a state's tables (evp_abi.cu with the two runtime calls replaced)
+    against copies that read their source only when the stream is waited for, which is
+    all that an asynchronous copy from pageable memory promises."""
+    from paper_1803_09563_gb300 import build
+    nvcc = build.nvcc()
+    if shutil.which(nvcc) is None:
+        pytest.skip('needs nvcc')
+    src = tmp_path / 'uploads.cu'
+    src.write_text(UPLOADS)
+    exe = tmp_path / 'uploads'
+    # the kernels' launchers live in other translation units and are not called
+    subprocess.run([nvcc, '-std=c++17', '-O1', '-I', CSRC, '-I', os.path.join(ROOT, 'include'), str(src), '-o', str(exe),
+                    '-Xlinker', '--unresolved-symbols=ignore-all'], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stdout, r.stderr)
