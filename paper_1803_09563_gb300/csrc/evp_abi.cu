@@ -1023,6 +1023,36 @@ cudaError_t copy_fields(const FieldCopies& c, int n, size_t bytes, cudaStream_t 
     return cudaGetLastError();
 }
 
+// May n fields of bytes each go to these buffers in one launch?  Everything the launch
+// touches lies on one device, the calling thread's current one, whose stream it runs on (a
+// copy call also reaches another device).  The copies run side by side: overlapping
+// destinations (or one inside the state's arena) keep their order with the copy calls, and
+// so do addresses below an element's alignment.
+bool one_launch(const evp_state* s, int n, void* const* dsts, size_t bytes) {
+    if (n < 2 || n > EVP_NFIELDS || bytes > GATHER_MAX) return false;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    auto here = [&](const void* p) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return at.type == cudaMemoryTypeDevice && at.device == dev;
+    };
+    const uintptr_t a = (uintptr_t)s->arena;
+    bool ok = here(s->arena);
+    for (int i = 0; ok && i < n; ++i) {
+        const uintptr_t d = (uintptr_t)dsts[i];
+        ok = d % 4 == 0 && !(d < a + s->arena_bytes && a < d + bytes) && here(dsts[i]);
+        for (int q = 0; ok && q < i; ++q) ok = !(d < (uintptr_t)dsts[q] + bytes && (uintptr_t)dsts[q] < d + bytes);
+    }
+    return ok;
+}
+
 int take_field(evp_state* s, int field, void* dst, int dst_on_device, cudaStream_t st) {
     CK(cudaMemcpyAsync(dst, field_ptr(s, field), s->N * s->elt,
                        dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
@@ -1080,23 +1110,7 @@ int evp_get_fields(evp_state* s, int n, const int* fields, void* const* dsts, in
         if (!field_ptr(s, fields[i])) return fail(EVP_ERR_ARG, "unknown field id");
     }
     const size_t bytes = s->N * s->elt;
-    bool gather = dst_on_device && n > 1 && n <= EVP_NFIELDS && bytes <= GATHER_MAX;
-    int dev = 0;
-    if (gather) CK(cudaGetDevice(&dev));
-    for (int i = 0; gather && i < n; ++i) {
-        // the copies run side by side: overlapping destinations (or one inside the state's
-        // arena) keep their order, and so do addresses below an element's alignment
-        const uintptr_t d = (uintptr_t)dsts[i], a = (uintptr_t)s->arena;
-        if (d % 4 != 0 || (d < a + s->arena_bytes && a < d + bytes)) gather = false;
-        for (int q = 0; q < i; ++q)
-            if (d < (uintptr_t)dsts[q] + bytes && (uintptr_t)dsts[q] < d + bytes) gather = false;
-        cudaPointerAttributes at;
-        if (gather && (cudaPointerGetAttributes(&at, dsts[i]) != cudaSuccess || at.type != cudaMemoryTypeDevice ||
-                       at.device != dev)) {
-            cudaGetLastError();
-            gather = false;
-        }
-    }
+    const bool gather = dst_on_device && one_launch(s, n, dsts, bytes);
     if (gather) {
         FieldCopies c;
         for (int i = 0; i < n; ++i) {
