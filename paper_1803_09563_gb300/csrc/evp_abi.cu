@@ -12,6 +12,7 @@
 #include "evp_internal.cuh"
 #include "evp_state.cuh"
 
+#include <cuda.h>
 #include <nvtx3/nvToolsExt.h>
 
 using namespace evp;
@@ -1023,11 +1024,29 @@ cudaError_t copy_fields(const FieldCopies& c, int n, size_t bytes, cudaStream_t 
     return cudaGetLastError();
 }
 
+// The device allocation that holds address p, from the driver (looked up at run time: the
+// library does not link it).  False where the driver cannot tell.
+bool allocation_of(uintptr_t p, uintptr_t* base, size_t* size) {
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess)
+            cudaGetLastError();
+        return found == cudaDriverEntryPointSuccess ? reinterpret_cast<Range>(f) : nullptr;
+    }();
+    CUdeviceptr b = 0;
+    if (!range || range(&b, size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    *base = (uintptr_t)b;
+    return true;
+}
+
 // May n fields of bytes each go to these buffers in one launch?  Everything the launch
 // touches lies on one device, the calling thread's current one, whose stream it runs on (a
 // copy call also reaches another device).  The copies run side by side: overlapping
 // destinations (or one inside the state's arena) keep their order with the copy calls, and
-// so do addresses below an element's alignment.
+// so do addresses below an element's alignment.  A buffer that ends beyond its allocation
+// goes to the copy calls too, which refuse it where a kernel would write past it.
 bool one_launch(const evp_state* s, int n, void* const* dsts, size_t bytes) {
     if (n < 2 || n > EVP_NFIELDS || bytes > GATHER_MAX) return false;
     int dev = 0;
@@ -1043,11 +1062,16 @@ bool one_launch(const evp_state* s, int n, void* const* dsts, size_t bytes) {
         }
         return at.type == cudaMemoryTypeDevice && at.device == dev;
     };
+    auto fits = [&](uintptr_t d) {
+        uintptr_t base = 0;
+        size_t size = 0;
+        return allocation_of(d, &base, &size) && d >= base && d - base <= size && bytes <= size - (d - base);
+    };
     const uintptr_t a = (uintptr_t)s->arena;
     bool ok = here(s->arena);
     for (int i = 0; ok && i < n; ++i) {
         const uintptr_t d = (uintptr_t)dsts[i];
-        ok = d % 4 == 0 && !(d < a + s->arena_bytes && a < d + bytes) && here(dsts[i]);
+        ok = d % 4 == 0 && !(d < a + s->arena_bytes && a < d + bytes) && here(dsts[i]) && fits(d);
         for (int q = 0; ok && q < i; ++q) ok = !(d < (uintptr_t)dsts[q] + bytes && (uintptr_t)dsts[q] < d + bytes);
     }
     return ok;

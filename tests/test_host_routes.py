@@ -14,6 +14,7 @@ CSRC = os.path.join(ROOT, 'paper_1803_09563_gb300', 'csrc')
 # arguments: the current device; then the state's arena and two destinations, each as
 # device, offset in its allocation and the allocation's bytes.  Prints 1 for one launch.
 PROGRAM = r'''
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <cstdlib>
@@ -33,6 +34,19 @@ static cudaError_t t_attr(cudaPointerAttributes* at, const void* p) {
     at->device = a ? a->dev : -2;
     return cudaSuccess;
 }
+static CUresult t_range(CUdeviceptr* base, size_t* size, CUdeviceptr p) {
+    const Alloc* a = find((uintptr_t)p);
+    if (!a) return CUDA_ERROR_INVALID_VALUE;
+    *base = a->base;
+    *size = a->size;
+    return CUDA_SUCCESS;
+}
+static cudaError_t t_entry(const char*, void** f, unsigned, unsigned long long, cudaDriverEntryPointQueryResult* r) {
+    *f = reinterpret_cast<void*>(&t_range);
+    *r = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
+#define cudaGetDriverEntryPointByVersion t_entry
 #define cudaGetDevice t_device
 #define cudaPointerGetAttributes t_attr
 #include "evp_abi.cu"
@@ -80,3 +94,11 @@ def route(tmp_path_factory):
     (1, 0, 1, 1, 0), (0, 0, 1, 1, 0), (0, 0, 0, 1, 0), (1, 0, 0, 0, 0)])
 def test_one_launch_only_on_one_device(route, cur, arena, a, b, want):
     assert route(cur, arena, (a, 0, BUF), (b, 256, BUF + 256)) == want
+
+
+# destinations that end with their allocation and one byte (or far) beyond it
+@pytest.mark.parametrize("a,b,want", [
+    ((0, BUF), (0, BUF), 1), ((512, BUF + 512), (0, BUF), 1), ((0, BUF - 1), (0, BUF), 0),
+    ((0, BUF), (0, BUF // 2), 0), ((0, BUF), (512, BUF), 0)])
+def test_one_launch_only_inside_the_allocations(route, a, b, want):
+    assert route(0, 0, (0,) + a, (0,) + b) == want
