@@ -413,8 +413,10 @@ __device__ __forceinline__ void stress_tile(const Geo<double>& g, const ModelCon
                 if (!fin) bits |= EVP_BIT_NONFINITE;
                 // trace limit and sign of det B: in single precision where its rounding (below
                 // 1e-6 of the sum of the terms' magnitudes) leaves no doubt, else in double
-                if (MODEL == EVP_FENE_P && !(s[0] + s[3] + s[5] < (1.0f - 1e-5f) * mc.f_L2)) {
-                    if (bn[0] + bn[3] + bn[5] >= mc.L2) bits |= EVP_BIT_TRACE_LIMIT;
+                if (MODEL == EVP_FENE_P) {
+                    const float tr32 = s[0] + s[3] + s[5], trm = fabsf(s[0]) + fabsf(s[3]) + fabsf(s[5]);
+                    if (!(fmaf(1e-6f, trm, tr32) < (1.0f - 1e-6f) * mc.f_L2) && bn[0] + bn[3] + bn[5] >= mc.L2)
+                        bits |= EVP_BIT_TRACE_LIMIT;
                 }
                 const float p35 = s[3] * s[5], p44 = s[4] * s[4], p15 = s[1] * s[5], p42 = s[4] * s[2], p14 = s[1] * s[4],
                             p32 = s[3] * s[2];

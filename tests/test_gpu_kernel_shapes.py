@@ -128,3 +128,17 @@ def test_level_set_chunks(evp, nx, ny, walls, prec):
         got.append(sim.get(evp.EVP_PHI))
     assert np.isfinite(got[0]).all() and not np.array_equal(got[0], phi.astype(got[0].dtype))
     assert np.array_equal(got[1], np.tile(got[0], (32, 1, 1)))
+
+
+# the trace limit of a B that is no longer positive definite: diagonals of 1e7 cancel to a
+# trace 0.1 above or 0.3 below L^2, less than a single-precision rounding of theirs
+@pytest.mark.parametrize("bzz,hit", [(59.7, True), (59.3, False)])
+def test_double_precision_trace_limit_of_cancelling_diagonals(evp, bzz, hit):
+    sim, st, g, prm = setup_case(evp, (36, 9, 8, True), 'fene_p', {'L2': 60.0}, evp.EVP_FP64)
+    full = lambda v: np.full(sim.shape, v)
+    sim.set_state(full(0.0), full(0.0), full(0.0), full(0.0),
+                  [full(v) for v in (1e7 + 0.4, 0.0, 0.0, -1e7, 0.0, bzz)])
+    sim.sync(raise_on_error=False)
+    sim.step(1e-24)
+    bits = sim.sync(raise_on_error=False)[1]
+    assert bool(bits & evp.EVP_BIT_TRACE_LIMIT) == hit
