@@ -373,9 +373,11 @@ int evp_diagnostics(evp_state* s, evp_diag* out);
  * conversion instructions, over all 2^32 binary32 patterns (widening) and 2^30
  * binary64 patterns around the binary32 range, including every kind of rounding
  * tie (narrowing).  Results must agree bit for bit, except that values in the
- * binary32 subnormal range give a signed zero and a NaN gives some NaN.
+ * binary32 subnormal range give a signed zero and a NaN gives some NaN.  Also the
+ * FP64 stress kernel's reciprocal, quotient and reciprocal square root against
+ * the rounded operations (2^24 operands each; 1, 1 and 3 ulps).
  * *mismatches receives the number of failures (0 expected).  Synchronous;
- * allocates 16 bytes.                                                          */
+ * allocates 24 bytes.                                                          */
 int evp_selftest(unsigned long long* mismatches);
 
 /* ---------------------------------------------------------------- batches

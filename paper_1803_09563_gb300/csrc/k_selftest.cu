@@ -1,10 +1,12 @@
 // Device self-test of the integer-operation conversions between binary32 and
 // binary64 (widen_f32, narrow_f64) against the conversion instructions: bit for
 // bit, except that binary32-subnormal values must come out as the signed zero and
-// a NaN as some NaN.
+// a NaN as some NaN; and of the refined reciprocal, quotient and reciprocal square root
+// (refined.cuh) against CUDA's rounded operations, within the bounds derived there.
 #include <algorithm>
 
 #include "evp_internal.cuh"
+#include "refined.cuh"
 
 namespace evp {
 
@@ -140,25 +142,56 @@ __global__ void k_selftest_narrow(unsigned long long* bad, unsigned per) {
     if (local) atomicAdd(bad, local);
 }
 
+__device__ __forceinline__ bool within_ulps(double a, double b, long long n) {
+    const long long q = __double_as_longlong(a) - __double_as_longlong(b);
+    return q <= n && -q <= n;
+}
+
+// random fractions and signs with exponents over the ranges of refined.cuh
+__global__ void k_selftest_refined(unsigned long long* bad, unsigned per) {
+    const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const double e_max = 0x1p-18;
+    unsigned long long local = 0;
+    for (unsigned q = 0; q < per; ++q) {
+        const unsigned long long id = t * per + q;
+        const unsigned long long r1 = splitmix64(3 * id), r2 = splitmix64(3 * id + 1), r3 = splitmix64(3 * id + 2);
+        auto value = [](unsigned long long r, unsigned long long biased) {
+            return __longlong_as_double((long long)((r & 0x800fffffffffffffull) | (biased << 52)));
+        };
+        // reciprocal: 2^-1020 .. 2^1020
+        const double d = value(r1, 3ull + r3 % 2041ull);
+        bool ok = within_ulps(rcp_refined(d), __drcp_rn(d), 1) && fabs(fma(-d, rcp_seed(d), 1.0)) <= e_max;
+        // quotient and reciprocal square root: 2^-500 .. 2^500
+        const double m = value(r1, 523ull + (r3 >> 12) % 1000ull), n = value(r2, 523ull + (r3 >> 24) % 1000ull);
+        ok = ok && refinable(m) && refinable(n) && within_ulps(div_refined(n, m), __ddiv_rn(n, m), 1);
+        const double x = fabs(m), y = rsqrt_seed(x);
+        // the rounded reference's own root costs it an ulp more
+        ok = ok && within_ulps(rsqrt_refined(x), __drcp_rn(__dsqrt_rn(x)), 3) && fabs(fma(-(x * y), y, 1.0)) <= e_max;
+        if (!ok) ++local;
+    }
+    if (local) atomicAdd(bad, local);
+}
+
 }  // namespace
 
 cudaError_t run_selftest(unsigned long long* mismatches) {
     unsigned long long* d = nullptr;
-    cudaError_t e = cudaMalloc(&d, 2 * sizeof(unsigned long long));
+    cudaError_t e = cudaMalloc(&d, 3 * sizeof(unsigned long long));
     if (e != cudaSuccess) return e;
-    e = cudaMemset(d, 0, 2 * sizeof(unsigned long long));
+    e = cudaMemset(d, 0, 3 * sizeof(unsigned long long));
     const unsigned per = 1024, threads = 256;
     const unsigned long long widen_threads = (1ull << 32) / per;             // 4 Mi threads: 2^32 patterns
     const unsigned narrow_blocks = 4096;                                      // 2^30 patterns
     if (e == cudaSuccess) {
         k_selftest_widen<<<(unsigned)(widen_threads / threads), threads>>>(d, per);
         k_selftest_narrow<<<narrow_blocks, threads>>>(d + 1, per);
+        k_selftest_refined<<<1024, threads>>>(d + 2, 64);                    // 2^24 operands
         e = cudaGetLastError();
     }
-    unsigned long long h[2] = {0, 0};
+    unsigned long long h[3] = {0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpy(h, d, sizeof(h), cudaMemcpyDeviceToHost);
     cudaFree(d);
-    *mismatches = h[0] + h[1];
+    *mismatches = h[0] + h[1] + h[2];
     return e;
 }
 

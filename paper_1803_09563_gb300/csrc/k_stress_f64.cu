@@ -21,6 +21,7 @@
 //     as much as an active one, and 32-wide tiles leave a quarter of the lanes idle
 //     on a 72-point row.
 #include "evp_internal.cuh"
+#include "refined.cuh"
 
 namespace evp {
 
@@ -40,28 +41,6 @@ __device__ __forceinline__ int pmod(int a, int n) {
     return r < 0 ? r + n : r;
 }
 
-// 1/d for a normal d: the hardware's approximation (relative error e about 2^-22) and
-// one third-order Newton step r (1 + e + e^2), e = 1 - d r, whose error is e^3
-__device__ __forceinline__ double rcp_refined(double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    e = fma(e, e, e);
-    return fma(r, e, r);
-}
-// n / d with one correction of the quotient by its remainder
-__device__ __forceinline__ double div_refined(double n, double d) {
-    const double r = rcp_refined(d), q = n * r;
-    return fma(fma(-d, q, n), r, q);
-}
-// 1/sqrt(x) for a normal x > 0: approximation and one third-order step
-// y (1 + e/2 + 3 e^2/8), e = 1 - x y^2
-__device__ __forceinline__ double rsqrt_refined(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 // x > 0 by integer compare (true for a positive NaN, whose products are NaN anyway)
 __device__ __forceinline__ bool positive_bits(double x) { return __double_as_longlong(x) > 0; }
@@ -79,7 +58,8 @@ __device__ __forceinline__ double smooth_a(double a) { return fma(a * (13.0 / 3.
 // field, ordered from far upwind: D_{-2}, D_{-1}, D_0, D_{+1}) from the upwind first
 // difference v3.  With e = -D the candidates are q_k = v3 + P_k/6,
 // P = (5 D_{-1} - 2 D_{-2}, D_{-1} + 2 D_0, 4 D_0 - D_{+1}); A1..A3 = smooth_a of the
-// third differences between neighbouring D.
+// third differences between neighbouring D.  The denominator is above 1e-21 and leaves
+// rcp_refined's range only where it is about to overflow (differences of B near 1e38).
 __device__ __forceinline__ double weno_shared(double dm2, double dm1, double d0, double dp1, double A1, double A2,
                                               double A3, double v3) {
     const double b1 = fma(3.0, dm1, -dm2), b2 = dm1 + d0, b3 = fma(3.0, d0, -dp1);
@@ -315,7 +295,8 @@ __device__ __forceinline__ void stress_tile(const Geo<double>& g, const ModelCon
                 F = 0.0;
                 av = 0.0;
             } else if (MODEL == EVP_FENE_P) {
-                F = div_refined(mc.L2, mc.L2 - (b0[0] + b0[3] + b0[5]));
+                const double d = mc.L2 - (b0[0] + b0[3] + b0[5]);
+                F = refinable(d) ? div_refined(mc.L2, d) : mc.L2 / d;
                 av = mc.a_fene;
             } else if (MODEL == EVP_SARAMITO) {
                 double gm = mc.gmod;
@@ -331,8 +312,11 @@ __device__ __forceinline__ void stress_tile(const Geo<double>& g, const ModelCon
                 double m2 = fma(d5, d5, fma(d3, d3, d0 * d0)) * 0.5;
                 m2 = fma(b0[4], b0[4], fma(b0[2], b0[2], fma(b0[1], b0[1], m2)));
                 const double mag2 = (gm * gm) * m2;
-                if (mag2 > 1e-290) {
+                if (refinable(mag2)) {
                     const double f = fma(-mc.tau_y, rsqrt_refined(mag2), 1.0);
+                    F = f > 0.0 ? f : 0.0;
+                } else if (mag2 > 0.0) {
+                    const double f = 1.0 - mc.tau_y / sqrt(mag2);
                     F = f > 0.0 ? f : 0.0;
                 } else {
                     F = mc.tau_y > 0.0 ? 0.0 : 1.0;
@@ -433,7 +417,8 @@ __device__ __forceinline__ void stress_tile(const Geo<double>& g, const ModelCon
                     // the divergence term of the momentum step
                     const double gm = mc.gmod;
                     if (MODEL == EVP_FENE_P) {
-                        const double Fn = div_refined(mc.L2, mc.L2 - (bn[0] + bn[3] + bn[5]));
+                        const double dn = mc.L2 - (bn[0] + bn[3] + bn[5]);
+                        const double Fn = refinable(dn) ? div_refined(mc.L2, dn) : mc.L2 / dn;
 #pragma unroll
                         for (int c = 0; c < 6; ++c) {
                             const double d = is_diag(c) ? mc.a_fene : 0.0;

@@ -142,3 +142,22 @@ def test_double_precision_trace_limit_of_cancelling_diagonals(evp, bzz, hit):
     sim.step(1e-24)
     bits = sim.sync(raise_on_error=False)[1]
     assert bool(bits & evp.EVP_BIT_TRACE_LIMIT) == hit
+
+
+# the closures where |tau^d|^2 overflows or is below the range of the refined reciprocal
+# square root, and where tr B = L^2 exactly, of a uniform B at rest: RT = (a I - F B)/lambda
+@pytest.mark.parametrize("model,extra,b,want", [
+    ('saramito', {'Bi': 0.4}, (1e160, 0.0, 0.0, 1.0, 0.0, 1.0), ((1.0 - 1e160) / 0.8, 0.0, 0.0, 0.0, 0.0, 0.0)),   # F = 1
+    ('saramito', {'Bi': 0.4}, (1.0, 1e-100, 0.0, 1.0, 0.0, 1.0), (0.0, 0.0, 0.0, 0.0, 0.0, 0.0)),                 # F = 0
+    ('saramito', {'Bi': 0.0}, (1.0, 1e-100, 0.0, 1.0, 0.0, 1.0), (0.0, -1e-100 / 0.8, 0.0, 0.0, 0.0, 0.0)),       # F = 1
+    ('fene_p', {'L2': 60.0}, (20.0, 1.0, 1.0, 20.0, 1.0, 20.0), (-np.inf,) * 6)])                                  # F = inf
+def test_double_precision_closures_at_the_ends_of_the_range(evp, model, extra, b, want):
+    import torch
+    sim, _, _, _ = setup_case(evp, (36, 9, 8, True), model, extra, evp.EVP_FP64)
+    z = np.zeros(sim.shape)
+    sim.set_state(z, z, z, z, [z + v for v in b])
+    out = torch.empty((6,) + sim.shape, dtype=torch.float64, device='cuda')
+    evp.evp_stress_rhs(sim.handle, out)
+    sim.sync(raise_on_error=False)
+    for c in range(6):
+        np.testing.assert_allclose(out[c].cpu().numpy(), z + want[c], rtol=1e-14, atol=0)
