@@ -43,13 +43,15 @@ def test_double_precision_stress_from_several_threads(evp, model, extra):
         s.sync()
         want.append(o.cpu().numpy())
 
-    def job(s, o):
+    lib = evp.load()
+
+    def job(s, p):
         def repeat():
-            for _ in range(1500):
-                evp.evp_stress_rhs(s.handle, o)
+            for _ in range(3000):          # the bare call: little else between a thread's launches
+                assert lib.evp_stress_rhs(s.handle, p) == 0, evp.evp_last_error()
             s.sync()
         return repeat
-    assert not in_threads([job(s, o) for s, o in zip(sims, outs)])
+    assert not in_threads([job(s, o.data_ptr()) for s, o in zip(sims, outs)])
     for w, o in zip(want, outs):
         assert np.array_equal(w, o.cpu().numpy())
 
