@@ -1062,16 +1062,22 @@ bool one_launch(const evp_state* s, int n, void* const* dsts, size_t bytes) {
         }
         return at.type == cudaMemoryTypeDevice && at.device == dev;
     };
-    auto fits = [&](uintptr_t d) {
-        uintptr_t base = 0;
-        size_t size = 0;
-        return allocation_of(d, &base, &size) && d >= base && d - base <= size && bytes <= size - (d - base);
+    // the allocation of the last buffer asked about: several buffers mostly share one
+    uintptr_t lo = 0, hi = 0;
+    auto fits = [&](void* p) {
+        const uintptr_t d = (uintptr_t)p;
+        if (d < lo || d >= hi) {
+            size_t size = 0;
+            if (!here(p) || !allocation_of(d, &lo, &size)) return false;
+            hi = lo + size;
+        }
+        return d >= lo && d < hi && bytes <= hi - d;
     };
     const uintptr_t a = (uintptr_t)s->arena;
     bool ok = here(s->arena);
     for (int i = 0; ok && i < n; ++i) {
         const uintptr_t d = (uintptr_t)dsts[i];
-        ok = d % 4 == 0 && !(d < a + s->arena_bytes && a < d + bytes) && here(dsts[i]) && fits(d);
+        ok = d % 4 == 0 && !(d < a + s->arena_bytes && a < d + bytes) && fits(dsts[i]);
         for (int q = 0; ok && q < i; ++q) ok = !(d < (uintptr_t)dsts[q] + bytes && (uintptr_t)dsts[q] < d + bytes);
     }
     return ok;

@@ -102,3 +102,10 @@ def test_one_launch_only_on_one_device(route, cur, arena, a, b, want):
     ((0, BUF), (0, BUF // 2), 0), ((0, BUF), (512, BUF), 0)])
 def test_one_launch_only_inside_the_allocations(route, a, b, want):
     assert route(0, 0, (0,) + a, (0,) + b) == want
+
+
+# two buffers of one allocation, the second ending with it and beyond it
+@pytest.mark.parametrize("extra,want", [(0, 1), (1, 0), (BUF, 0)])
+def test_one_launch_with_two_buffers_of_one_allocation(route, extra, want):
+    # the program puts allocation q at (q + 1) 2^40: the third buffer's offset reaches back
+    assert route(0, 0, (0, 0, 2 * BUF), (0, BUF + extra - (1 << 40), BUF)) == want
