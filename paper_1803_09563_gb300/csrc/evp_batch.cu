@@ -117,14 +117,14 @@ bool find_config(const evp_grid& g, int precision, int model, evp_tile_config* o
 // rules (k_stress.cuh, k_momentum.cu) on the whole launch's items, so that the small grids
 // of a batch are not cut into one-plane items (each with the start of a chunk) for an SM
 // count that the batch fills many times over.  start: what an SM pays beside its items.
-int batch_planes(const std::vector<std::pair<int, int>>& tiles_nz, double start) {
+int batch_planes(const std::vector<std::pair<int, int>>& tiles_nz, double start, int sms) {
     int best = 1, most = 1;
     for (const auto& t : tiles_nz) most = std::max(most, t.second);
     double cost = -1.0;
     for (int kz = 1; kz <= most && kz <= 64; ++kz) {
         long long items = 0;
         for (const auto& t : tiles_nz) items += (long long)t.first * ((t.second + kz - 1) / kz);
-        const double c = ((items + 151) / 152 + start) * (kz + 1);
+        const double c = ((items + sms - 1) / sms + start) * (kz + 1);
         if (cost < 0.0 || c <= cost) {
             cost = c;
             best = kz;
@@ -290,7 +290,7 @@ int prepare(evp_batch* b) {
             const auto n = grid_of(b->m[i].s->g);
             t.emplace_back(n.first * n.second, b->m[i].s->g.nz);
         }
-        const int kz = batch_planes(t, start);
+        const int kz = batch_planes(t, start, sms);
         for (int i : idx)
             if (!b->m[i].own_cfg) b->m[i].cfg.*field = std::min(kz, b->m[i].s->g.nz);
     };

@@ -174,3 +174,46 @@ def test_autotuner_matches_exhaustive_sweep(evp):
     assert min(tq) <= 1.10 * min(tf) + 0.005, (quick.as_tuple(), full.as_tuple(), tq, tf)
     # the table keeps the last tuning of this grid
     assert evp.evp_tile_config_get(grid, evp.EVP_FP32, 'saramito').as_tuple() == full.as_tuple()
+
+
+# seven grids in two models: more Poisson chains than streams (the sixth and seventh queue
+# behind the first and second), rows staged in 16-byte chunks (nx % 4 == 0) beside rows
+# staged by element (18, 54, 162), so that both the stress and the momentum phase have
+# launches beside one another
+MANY = [
+    (32, 32, 32, False, 'saramito', {'Bi': 0.4}),
+    (18, 12, 24, True, 'saramito', {'Bi': 0.4}),
+    (54, 18, 16, False, 'oldroyd_b', {}),
+    (64, 12, 24, True, 'oldroyd_b', {}),
+    (48, 24, 18, False, 'saramito', {'Bi': 0.2}),
+    (162, 9, 8, True, 'oldroyd_b', {}),
+    (36, 20, 16, True, 'saramito', {'Bi': 0.4}),
+]
+
+
+@pytest.mark.parametrize('prec', ['fp32', 'fp64'])
+@pytest.mark.parametrize('graph', [False, True])
+def test_batch_of_many_grids_equals_each_member_alone_bitwise(evp, prec, graph):
+    precision = evp.EVP_FP32 if prec == 'fp32' else evp.EVP_FP64
+    want = []
+    for i, case in enumerate(MANY):
+        sim = member(evp, case, precision, 90 + 3 * i)
+        for _ in range(3):
+            sim.step(1e-3)
+        sim.sync()
+        want.append(snapshot(evp, sim))
+        sim.close()
+    batch = evp.Batch(precision)
+    evp.evp_batch_set_graph(batch.handle, graph)
+    sims = [member(evp, case, precision, 90 + 3 * i) for i, case in enumerate(MANY)]
+    for sim in sims:
+        batch.admit(sim, 1e-3)
+    for _ in range(3):
+        batch.step()
+    for i, sim in enumerate(sims):
+        assert sim.sync(raise_on_error=False)[0] == 0
+        for a, b in zip(want[i], snapshot(evp, sim)):
+            assert np.array_equal(a, b), (i, MANY[i][:5])
+    batch.close()
+    for sim in sims:
+        sim.close()
