@@ -161,3 +161,29 @@ def test_double_precision_closures_at_the_ends_of_the_range(evp, model, extra, b
     sim.sync(raise_on_error=False)
     for c in range(6):
         np.testing.assert_allclose(out[c].cpu().numpy(), z + want[c], rtol=1e-14, atol=0)
+
+
+# chunks of three planes and more with a short last one, by the chunk rules themselves: 32 x
+# 8 momentum tiles staged by element (nx % 4 = 2) and in 16-byte chunks, 64 x 4 tiles, walls
+# (planes whose ghost rows are set inside the march) and none, the double-precision kernels
+@pytest.mark.parametrize("shape,prec", [
+    ((18, 33, 64, True), 1), ((36, 33, 32, True), 1), ((36, 36, 32, False), 1), ((64, 17, 64, True), 1),
+    ((128, 33, 54, True), 1), ((18, 29, 64, True), 0), ((36, 33, 32, True), 0), ((72, 36, 54, False), 0)])
+@pytest.mark.parametrize("model,extra", [('saramito', {'Bi': 0.4}), ('newtonian', {})])
+def test_chunks_with_a_remainder(evp, shape, prec, model, extra):
+    sim, st, g, prm = setup_case(evp, shape, model, extra, prec, dpdx=0.3)
+    cfg = evp.evp_tile_config_get(sim.grid, prec, model)
+    for kz in (cfg.stress_kz, cfg.momentum_kz):
+        assert kz > 2 and shape[2] % kz, kz
+    # a quarter of the explicit viscous limit dt 4 mu_s sum 1/h^2 <= 2.51
+    h2 = sum((n / l) ** 2 for n, l in zip(shape[:3], (g.lx, g.ly, g.lz)))
+    dt = min(1e-3, 0.25 * 2.51 / (4 * 0.4 / 2.0 * h2))
+    for _ in range(2):
+        sim.step(dt)
+        st = oracle.rk3_step(st, dt, g, prm, force=(0.3, 0.0, 0.0))
+    sim.sync()
+    pairs = [(evp.EVP_U, st.U), (evp.EVP_V, st.V), (evp.EVP_W, st.W)]
+    if model != 'newtonian':
+        pairs += [(evp.EVP_BXX + c, st.B[c]) for c in range(6)]
+    for f, ref in pairs:
+        assert rel(sim.get(f), ref) < (1e-5 if prec else 1e-10), (f, rel(sim.get(f), ref))
