@@ -399,8 +399,9 @@ typedef struct evp_batch_s evp_batch;
 
 /* Tile configuration of the batched kernels for one grid: z planes per work item
  * of the stress and momentum kernels, resident CTAs per SM of their persistent
- * grids (at most 2 and 4 in FP32, 1 and 2 in FP64), and kx columns per block of
- * the column FFT passes (4, 8 or 16; 16 only in FP32).  0 in a field: the
+ * grids (at most 2 and 4 in FP32, counted in CTAs of 256 threads; 1 and 2 in
+ * FP64, where a count stands for two CTAs of 128 threads), and kx columns per block
+ * of the column FFT passes (4, 8 or 16; 16 only in FP32).  0 in a field: the
  * default (the heuristic of the single-state launches).  A batch of several FP32
  * members sizes the work items of grids without an entry for the whole batch.  */
 typedef struct {
