@@ -273,8 +273,8 @@ __device__ __forceinline__ void momentum_point(const Geo<T>& g, const ModelConst
 // the same kernel without its arithmetic 232, a plain stream over the same 19 arrays 164
 // and the arithmetic on planes already there 210; deeper staging (a fourth slot, fewer
 // CTAs), L1-allocating copies, tiles of 128 columns and reading the neighbours straight
-// through L1 were slower (288, 308, 285, 319 us).  The kernel before this one, with one
-// ring per field and the fluxes through the lower faces computed again, took 289 us.
+// through L1 were slower (288, 308, 285, 319 us), and so were one ring per field with the
+// fluxes through the lower faces computed again (289 us).
 template <int TX_, int TY_>
 struct MomTile {
     static constexpr int TX = TX_, TY = TY_, NT = TX * TY;

@@ -552,15 +552,15 @@ __device__ __forceinline__ void momentum_ab2_cell(const Geo<T>& g, const MomAB2A
     a.NH[2][c0] = Nz;
 }
 
-// z-marching tiles of the AB2 momentum step: a 32 x 4 tile walks a chunk of z planes.  Planes k-1, k, k+1 of u, v, w, H and tau (built once per staged cell
-// from B^n and H, instead of once per stencil use) and planes k, k+1 of the
-// interface force sit in shared memory with a one-cell halo in x and y, staged
-// with the periodic wraps and the wall ghost rules; the raw values of plane k+2
-// are loaded into registers before plane k is computed.  A staged cell's offset and its
-// wall ghost (the nearest row, u and w negated, v zero) are found once per thread.
-// Bound by instruction issue and shared-memory reads, about 45 a cell.  128 x 256 x 128 FP32:
-// 154 us with wraps and ghost rules at each of the 13 reads of a staged cell, 146 so
-// (32 x 8 tiles 150, 32 x 16 160).
+// z-marching tiles of the AB2 momentum step: a 32 x 4 tile walks a chunk of z planes.
+// Planes k-1, k, k+1 of u, v, w, H and tau (built once per staged cell from B^n and H,
+// instead of once per stencil use) and planes k, k+1 of the interface force sit in
+// shared memory with a one-cell halo in x and y, staged with the periodic wraps and the
+// wall ghost rules; the raw values of plane k+2 are loaded into registers before plane k
+// is computed.  A staged cell's offset and its wall ghost (the nearest row, u and w
+// negated, v zero) are found once per thread.  Bound by instruction issue and
+// shared-memory reads, about 45 a cell.  128 x 256 x 128 FP32: 154 us with wraps and ghost
+// rules at each of the 13 reads of a staged cell, 144 so (32 x 8 tiles 150, 32 x 16 160).
 constexpr int AB_TX = 32, AB_TY = 4, AB_NT = AB_TX * AB_TY;
 constexpr int AB_W = AB_TX + 2, AB_PL = AB_W * (AB_TY + 2);
 constexpr int AB_NE = (AB_PL + AB_NT - 1) / AB_NT;          // staged cells per thread
