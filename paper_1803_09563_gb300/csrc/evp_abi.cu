@@ -1027,8 +1027,8 @@ cudaError_t copy_fields(const FieldCopies& c, int n, size_t bytes, cudaStream_t 
     return cudaGetLastError();
 }
 
-// The device allocation that holds address p, from the driver (looked up at run time: the
-// library does not link it).  False where the driver cannot tell.
+// The device allocation that holds address p, from the CUDA driver API (looked up at run
+// time: the library does not link libcuda).  False where it cannot tell.
 bool allocation_of(uintptr_t p, uintptr_t* base, size_t* size) {
     using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
     static const Range range = [] {
